@@ -23,6 +23,8 @@
 // (CP) terms.  A level's local lists are complete when its walk kernel ends, so a large walk runs
 // their M2L and P2L terms and the level's top-down pass on a side stream while the walk goes on
 // below; a small one runs them after its last level.
+#include <limits.h>
+
 #include <algorithm>
 
 #include "expansions.cuh"
@@ -32,18 +34,14 @@
 #define WALK_WPB 4
 #define WALK_THREADS (WALK_WPB * 32)
 
-enum { OUT_NONE = 0, OUT_ACCEPT = 1, OUT_DEFER = 2, OUT_PC = 3, OUT_PP = 4, OUT_OPEN = 5 };
-
-// Learned criterion (MODE 1): the pairs the network must decide are not evaluated one step at a
-// time, where a step has a few of them and the tensor-core tile of 16 rows runs mostly empty.  They
-// wait in a per-warp buffer (entry and features) until 32 of them fill two tiles, or the sink's
-// queue runs dry; the evaluated entries return to the queue marked with their decision, and the
-// next steps sort them like any other entry.  Marks: bit 30 accepted, bit 29 rejected (cell entries
-// of an isolated box, whose indices stay below 2^29).
+// Learned criterion (MODE 1): the pairs the network must decide wait in a list of the sink's until
+// its queue runs dry.  They are then evaluated 32 per warp, which fills two tensor-core tiles, and
+// return to the queue in the order they were met, marked with their decision; the next steps sort
+// them like any other entry.  So the order of the queue does not depend on how many entries a step
+// takes.  Marks: bit 30 accepted, bit 29 rejected (cell entries of an isolated box, whose indices
+// stay below 2^29).
 #define WALK_NET_ACC (1u << 30)
 #define WALK_NET_REJ (1u << 29)
-#define WALK_PEND 64  // pending pairs per warp: fewer than 32 left after a flush, plus one step's 32
-#define WALK_PEND_BYTES (WALK_PEND * 4 + WALK_PEND * MLP_F * 4)
 
 __device__ __forceinline__ float d2_ordered(float dx, float dy, float dz)
 {
@@ -57,453 +55,472 @@ __device__ __forceinline__ float gap_axis(float lo_s, float hi_s, float lo_k, fl
     return g > 0.0f ? g : 0.0f;
 }
 
-// MODE 0: fixed-theta criterion.  MODE 1: learned criterion for source cells (the network
-// decides inside the band, see mlp.cuh).  MODE 2: fixed criterion, and every (sink, source cell)
-// pair of the band is recorded for labelling (audit).
-//
-// A warp examines up to E * 32 entries of its sink's queue per step: lane l takes entries
-// base + s * 32 + l for slots s < E, the loads of every slot are in flight together, and the
-// outcomes are ranked slot by slot, so each list comes out in queue order, exactly as with one
-// entry per lane.  A sink's serial chain of steps (its checklist and what it opens, 32 entries
-// at a time) set each level's duration; E entries per lane shorten it E-fold where the queue is
-// long, and cost nothing extra where it is short (slots past the queue are skipped, warp-uniformly).
-//
-// Measured on the 128^3 NFW box: 2 to 4 entries per lane made the walk slower (3.93 ms with one,
-// 4.09 with two, 4.41 with four), because the extra registers halve the resident warps and each
-// entry's chain of dependent instructions does not shorten; one entry per lane is the default.
-#ifndef FMM_WALK_SLOTS
-#define FMM_WALK_SLOTS 1  // entries per lane and step
-#endif
+// Resident blocks per SM the fixed-theta walk is compiled for: 6 (80 registers, all of the grid's 24
+// warps per SM resident) against 5, walk phase 3.04 against 3.08 ms on the 128^3 NFW box and 15.5
+// against 16.1 ms on a 256^3 box with a tenth of its particles active.
 #ifndef FMM_WALK_MINB
-#define FMM_WALK_MINB 5  // resident blocks per SM the fixed-theta walk is compiled for (96 registers, no spills)
+#define FMM_WALK_MINB 6
 #endif
-template <int MODE>
-struct WalkSlots {
-    static constexpr int E = FMM_WALK_SLOTS;
+// A level of fewer than FMM_WALK_TEAM_SINKS sinks per block of the grid gives every sink a whole
+// block (walk_sinks).  Walk phase by this line, 128^3 NFW box / 200^3 box with the learned
+// criterion: 1: 3.54 / 11.8 ms, 2: 3.21 / 11.8, 4: 3.08 / 11.7, 8: 3.11 / 11.7, 16: 3.23 / 11.8,
+// every level: 3.22 / 13.9.
+#ifndef FMM_WALK_TEAM_SINKS
+#define FMM_WALK_TEAM_SINKS 4
+#endif
+
+// What a walk level reads and writes (one kernel parameter).
+struct WalkIO {
+    const WalkNode* node;
+    const float4* posf;
+    const int* cnact;
+    const int* f_cell;
+    const unsigned long long* f_cloff;
+    const int* f_cllen;
+    const unsigned int* cl_cur;
+    int* f_cell_next;
+    unsigned long long* f_cloff_next;
+    int* f_cllen_next;
+    unsigned int* cl_next;
+    unsigned long long *lcc_off, *lcp_off;
+    int *lcc_len, *lcp_len, *wcells;
+    unsigned int *pp, *pc, *cc, *cp;
+    int *cc_sink, *cp_sink;
+    Group* groups;
+    unsigned int* scratch;
+    DevCounters* ctr;
+    long long cap_front, cap_cl, cap_pp, cap_pc, cap_cc, cap_cp, cap_groups, cap_scr;
+    int level, group;
+    float four_eps2;
+    // learned criterion and audit
+    const float4* mnorm;
+    const float* amin;
+    float eps, band_lo, band_hi, tau, margin;
+    const unsigned char* mlp_packed;
+    int2* audit_pairs;
+    long long audit_cap;
+    const unsigned char* nogroup;
+    PeriodicArgs pa;
 };
 
-// PER: a periodic box (list entries carry a copy code above their index bits); the isolated walk is
-// compiled without the decoding.
-template <int MODE, bool PER>
-__global__ void __launch_bounds__(WALK_THREADS, MODE == 1 ? 4 : FMM_WALK_MINB) k_walk_level(
-    const WalkNode* __restrict__ node, const float4* __restrict__ posf, const int* __restrict__ cnact,
-    const int* __restrict__ f_cell, const unsigned long long* __restrict__ f_cloff, const int* __restrict__ f_cllen,
-    int level, const unsigned int* __restrict__ cl_cur, int* __restrict__ f_cell_next,
-    unsigned long long* __restrict__ f_cloff_next, int* __restrict__ f_cllen_next, long long cap_front,
-    unsigned int* __restrict__ cl_next, long long cap_cl, unsigned long long* __restrict__ lcc_off,
-    int* __restrict__ lcc_len, unsigned long long* __restrict__ lcp_off, int* __restrict__ lcp_len,
-    int* __restrict__ wcells,
-    unsigned int* __restrict__ pp, long long cap_pp, unsigned int* __restrict__ pc,
-    long long cap_pc, unsigned int* __restrict__ cc, int* __restrict__ cc_sink, long long cap_cc,
-    unsigned int* __restrict__ cp, int* __restrict__ cp_sink, long long cap_cp,
-    Group* __restrict__ groups, long long cap_groups, unsigned int* __restrict__ scratch, long long cap_scr,
-    DevCounters* __restrict__ ctr, int bucket, int group, float four_eps2, const float4* __restrict__ mnorm,
-    const float* __restrict__ amin,
-    float eps, float band_lo, float band_hi, float tau, float margin, const unsigned char* __restrict__ mlp_packed,
-    int2* __restrict__ audit_pairs, long long audit_cap, const unsigned char* __restrict__ nogroup, PeriodicArgs pa)
+// A team's shared words: the counts of every warp's step (two steps' worth), and broadcasts.
+struct WalkShared {
+    uint2 cnt[2][WALK_WPB];
+    unsigned int srcpp;
+    unsigned long long fi, at[5];
+};
+
+// Barrier of the TEAM warps that share a sink: the warp itself, or the whole block.
+template <int TEAM>
+__device__ __forceinline__ void team_sync()
 {
-    constexpr int E = WalkSlots<MODE>::E;
-    const unsigned int q0 = PER ? copy_centre(pa.R) : 0u;
-    const int ib = PER ? pa.ib : 31;  // index bits of a list entry
-    extern __shared__ __align__(16) unsigned char walk_smem[];
-    if (MODE == 1) {
-        mlp_load_smem(mlp_packed, walk_smem);
-        __syncthreads();
+    if (TEAM == 1) __syncwarp();
+    else __syncthreads();
+}
+
+// A source as the criterion sees it: a cell's node, or a particle as a node of no extent.  A
+// source in a periodic copy has its centre and box shifted in FP64, then rounded, read from the
+// tables of those values (the axes with a non-zero shift).
+template <bool PER>
+__device__ __forceinline__ WalkNode walk_source(const WalkIO& w, unsigned int e, unsigned int q0, int ib)
+{
+    const unsigned int j = entry_index(e, ib);
+    const bool part = (e & FMM_PARTICLE_BIT) != 0u;
+    WalkNode S;
+    const float4* src = part ? w.posf + j : reinterpret_cast<const float4*>(w.node + j);
+    S.a = __ldg(src);
+    if (!part) {
+        S.b = __ldg(src + 1);
+        S.c = __ldg(src + 2);
+        S.d = __ldg(reinterpret_cast<const int4*>(src + 3));
+    } else {
+        S.d = make_int4(-1, -1, 0, 1);
     }
-    unsigned char* mlp_scratch = walk_smem + MLPP_SIZE + (threadIdx.x >> 5) * MLP_WARP_SCRATCH;
-    unsigned int* pend_e = reinterpret_cast<unsigned int*>(walk_smem + MLPP_SIZE + WALK_WPB * MLP_WARP_SCRATCH +
-                                                           (threadIdx.x >> 5) * WALK_PEND_BYTES);
-    float* pend_f = reinterpret_cast<float*>(pend_e + WALK_PEND);
-    static_assert(MODE != 1 || E == 1, "the learned walk takes one entry per lane and step");
-    unsigned long long n_mlp = 0;
-    const int lane = threadIdx.x & 31;
-    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    unsigned int* Q = scratch + gw * 5 * cap_scr;
-    unsigned int* D = Q + cap_scr;
-    unsigned int* A = Q + 2 * cap_scr;  // accepted: multipole sources from the front, point sources from the back
-    unsigned int* P = Q + 3 * cap_scr;
-    unsigned int* C = Q + 4 * cap_scr;
+    if (PER && entry_copy(e, ib) != q0) {
+        int nv[3];
+        copy_shift(entry_copy(e, ib), w.pa.R, nv[0], nv[1], nv[2]);
+        const int w2 = 2 * w.pa.R;
+#pragma unroll
+        for (int ax = 0; ax < 3; ax++) {
+            if (nv[ax] == 0) continue;
+            const long long slot = ((long long)j * 3 + ax) * w2 + shift_slot(nv[ax], w.pa.R);
+            float4 g;
+            if (part) g.x = w.pa.pshift[slot];
+            else g = w.pa.cshift[slot];
+            if (ax == 0) {
+                S.a.x = g.x;
+                S.b.x = g.y;
+                S.c.x = g.z;
+            } else if (ax == 1) {
+                S.a.y = g.x;
+                S.b.y = g.y;
+                S.c.y = g.z;
+            } else {
+                S.a.z = g.x;
+                S.b.z = g.y;
+                S.c.z = g.z;
+            }
+        }
+    }
+    if (part) {
+        S.a.w = 0.0f;
+        S.b = S.c = S.a;
+    }
+    return S;
+}
+
+// The sinks of one level.  TEAM warps share a sink (1: every warp has its own; WALK_WPB: the whole
+// block) and examine 32 * TEAM entries of its queue per step, one per lane.  Outcomes are ranked in
+// queue order (ballots within a warp, the warps' counts through shared memory), so the lists and
+// the queue come out in the same order whatever TEAM is.
+//
+// A step is a chain of a few hundred dependent instructions and two dependent loads (the entry, its
+// node), 1.4 us with one warp per sink; a level lasts as long as its longest sink's chain of steps
+// (up to 170 on the 128^3 NFW box) unless its sinks fill the GPU.  So a level of few sinks takes
+// TEAM = WALK_WPB, which cuts every chain by that factor, and a full level takes TEAM = 1, which has
+// no barriers and wastes fewer lanes on the ends of queues.  Walk phase with local expansions, one
+// warp per sink on every level against this: 4.38 to 3.04 ms on the 128^3 NFW box, 2.04 to 1.24 ms
+// on a 63^3 one, 0.49 to 0.37 ms on a 4096-particle box, 2.55 to 1.31 ms on a dual-tree substep.
+//
+// MODE 0: fixed-theta criterion.  MODE 1: learned criterion for source cells (the network
+// decides inside the band, see mlp.cuh).  MODE 2: fixed criterion, and every (sink, source cell)
+// pair of the band is recorded for labelling (audit).  PER: a periodic box (list entries carry a
+// copy code above their index bits); the isolated walk is compiled without the decoding.
+template <int MODE, bool PER, int TEAM>
+__device__ __forceinline__ void walk_sinks(const WalkIO& w, const unsigned long long n_front,
+                                           const unsigned long long wbase, WalkShared& sh,
+                                           const unsigned char* walk_smem, unsigned char* mlp_scratch)
+{
+    constexpr int WIN = 32 * TEAM;
+    const unsigned int q0 = PER ? copy_centre(w.pa.R) : 0u;
+    const int ib = PER ? w.pa.ib : 31;  // index bits of a list entry
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    const int tl = TEAM == 1 ? lane : (int)threadIdx.x;  // position in the team
+    const int tw = TEAM == 1 ? 0 : wl;                   // warp of the team
+    const int cap = (int)min(w.cap_scr * TEAM, (long long)INT_MAX);
+    DevCounters* const ctr = w.ctr;
+    // the team's scratch: queue, deferred, accepted (multipole sources from the front, point sources
+    // from the back), PP and PC entries; pairs for the network wait in the list that the sink leaves
+    // unused (a group defers nothing, any other sink has no PP entries)
+    unsigned int* const Q = w.scratch + ((long long)blockIdx.x * WALK_WPB + (TEAM == 1 ? wl : 0)) * 5 * w.cap_scr;
+    unsigned int* const D = Q + w.cap_scr * TEAM;
+    unsigned int* const A = D + w.cap_scr * TEAM;
+    unsigned int* const P = A + w.cap_scr * TEAM;
+    unsigned int* const C = P + w.cap_scr * TEAM;
     const unsigned int lt = fmm_lanemask_lt();
-    const unsigned long long n_front = *(volatile unsigned long long*)&ctr->lv_front[level];
-    // this level's sinks go to the walked-cell list after the levels before it
-    const unsigned long long wbase = *(volatile unsigned long long*)&ctr->lv_base[level];
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctr->lv_base[level + 1] = wbase + n_front;
-    unsigned long long w_entries = 0, w_max = 0;  // this warp's statistics, added once at the end
+    unsigned long long w_entries = 0, n_mlp = 0;  // this team's statistics, added once at the end
+    int w_max = 0;
 
     for (;;) {
         unsigned long long fi = 0;
-        if (lane == 0) fi = atomicAdd(&ctr->lv_work[level], 1ull);
-        fi = __shfl_sync(FMM_FULL_MASK, fi, 0);
+        if (TEAM == 1) {
+            if (lane == 0) fi = atomicAdd(&ctr->lv_work[w.level], 1ull);
+            fi = __shfl_sync(FMM_FULL_MASK, fi, 0);
+        } else {
+            __syncthreads();  // the last sink's shared words are done with
+            if (threadIdx.x == 0) {
+                sh.fi = atomicAdd(&ctr->lv_work[w.level], 1ull);
+                sh.srcpp = 0u;
+            }
+            __syncthreads();
+            fi = sh.fi;
+        }
         if (fi >= n_front) break;
-        const int k = f_cell[fi];
-        if (lane == 0 && (long long)(wbase + fi) < cap_front) wcells[wbase + fi] = k;
-        const WalkNode K = node[k];
+        const int k = w.f_cell[fi];
+        if (tl == 0 && (long long)(wbase + fi) < w.cap_front) w.wcells[wbase + fi] = k;
+        const WalkNode K = w.node[k];
         // a group holds <= g particles; in a graded tree (dual trees) it is also no larger than the
         // fixed tree's groups around it
-        const bool kg = K.d.w <= group && !(nogroup && nogroup[k]);
-        const float rk = K.a.w, bk = K.b.w;
-        const float ak = MODE == 1 ? amin[k] : 0.0f;
-        const unsigned long long cl0 = f_cloff[fi];
-        const long long ncl = f_cllen[fi];
-        long long nq = 0, nd = 0, na = 0, nap = 0, npp = 0, npc = 0;
-        int npend = 0;  // learned criterion: pairs waiting for the network
+        const bool kg = K.d.w <= w.group && !(w.nogroup && w.nogroup[k]);
+        const float rk = K.a.w, bk = K.b.w, rk15 = __fmul_rn(1.5f, rk);
+        const float ak = MODE == 1 ? w.amin[k] : 0.0f;
+        const unsigned int* const cl = w.cl_cur + w.f_cloff[fi];
+        const int ncl = w.f_cllen[fi];
+        unsigned int* const X = kg ? C : D;  // a group's PC entries, any other sink's deferred ones
+        unsigned int* const W = kg ? D : P;  // pairs for the network (MODE 1)
+        int total = ncl, na = 0, nap = 0, nx = 0, npp = 0, nw = 0;
+        int base = 0, par = 0;
         int srcpp = 0;  // this lane's PP source particles
         bool overflow = false;
-        long long base = 0;
-        while (base < ncl + nq) {
-            // entries appended while this step runs get indices >= ncl + nq (step start), so the
-            // next step begins right after the entries that were actually available here
-            const long long avail = ncl + nq - base;
-            const int ns = avail >= 32 * E ? E : (int)((avail + 31) >> 5);  // slots in use (warp-uniform)
-            unsigned int e[E];
-            bool valid[E];
-#pragma unroll
-            for (int s = 0; s < E; s++) {
-                const long long vi = base + s * 32 + lane;
-                valid[s] = s < ns && s * 32 + lane < avail;
-                e[s] = 0;
-                if (valid[s]) e[s] = vi < ncl ? cl_cur[cl0 + vi] : Q[vi - ncl];
-            }
-            unsigned int decided = 0u;  // learned criterion: the network's decision carried by the entry
-            if (MODE == 1 && valid[0] && !(e[0] & FMM_PARTICLE_BIT)) {
-                decided = e[0] & (WALK_NET_ACC | WALK_NET_REJ);
-                e[0] &= ~(WALK_NET_ACC | WALK_NET_REJ);
-            }
-            base += avail < 32 * E ? avail : 32 * E;
-            WalkNode S[E];
-#pragma unroll
-            for (int s = 0; s < E; s++) {
-                if (valid[s]) {
-                    const unsigned int j = entry_index(e[s], ib);
-                    if (e[s] & FMM_PARTICLE_BIT) S[s].a = posf[j];
-                    else S[s] = node[j];
+        for (;;) {
+            while (base < total) {
+                const int vi = base + tl;
+                bool valid = vi < total;
+                unsigned int e = 0u;
+                if (valid) e = vi < ncl ? cl[vi] : Q[vi - ncl];
+                base = min(base + WIN, total);  // entries appended by this step follow
+                unsigned int decided = 0u;  // learned criterion: the network's decision carried by the entry
+                if (MODE == 1 && !(e & FMM_PARTICLE_BIT)) {
+                    decided = e & (WALK_NET_ACC | WALK_NET_REJ);
+                    e &= ~(WALK_NET_ACC | WALK_NET_REJ);
                 }
-            }
-            // a source in a periodic copy: its centre and box shifted in FP64, then rounded, read from
-            // the tables of those values (the axes with a non-zero shift)
-#pragma unroll
-            for (int s = 0; s < E; s++) {
-                if (PER && valid[s] && entry_copy(e[s], ib) != q0) {
-                    const unsigned int j = entry_index(e[s], ib);
-                    int nv[3];
-                    copy_shift(entry_copy(e[s], ib), pa.R, nv[0], nv[1], nv[2]);
-                    const int w2 = 2 * pa.R;
-#pragma unroll
-                    for (int ax = 0; ax < 3; ax++) {
-                        if (nv[ax] == 0) continue;
-                        const long long slot = ((long long)j * 3 + ax) * w2 + shift_slot(nv[ax], pa.R);
-                        if (e[s] & FMM_PARTICLE_BIT) {
-                            const float x = pa.pshift[slot];
-                            if (ax == 0) S[s].a.x = x;
-                            else if (ax == 1) S[s].a.y = x;
-                            else S[s].a.z = x;
-                        } else {
-                            const float4 g = pa.cshift[slot];
-                            if (ax == 0) {
-                                S[s].a.x = g.x;
-                                S[s].b.x = g.y;
-                                S[s].c.x = g.z;
-                            } else if (ax == 1) {
-                                S[s].a.y = g.x;
-                                S[s].b.y = g.y;
-                                S[s].c.y = g.z;
-                            } else {
-                                S[s].a.z = g.x;
-                                S[s].b.z = g.y;
-                                S[s].c.z = g.z;
-                            }
-                        }
-                    }
-                }
-            }
-            int out[E], nadd[E], sfirst[E], c0[E], c1[E], nsrc_cell[E];
-            bool sleaf[E], ptl[E];
-#pragma unroll
-            for (int s = 0; s < E; s++) {
-                out[s] = OUT_NONE;
-                nadd[s] = 0;
-                sfirst[s] = 0;
-                c0[s] = c1[s] = -1;
-                nsrc_cell[s] = 0;
-                sleaf[s] = false;
-                ptl[s] = false;
-                if (s >= ns) continue;
-                float f[MLP_F];  // learned criterion: the pair's features (set for band pairs)
-                bool pointlike = false, acc = false, need = false;
-                float d2 = 0.0f, ro = 0.0f;
-                if (valid[s]) {
-                    float cx, cy, cz, lox, loy, loz, hix, hiy, hiz;
-                    if (e[s] & FMM_PARTICLE_BIT) {
-                        const float4 p = S[s].a;
-                        cx = lox = hix = p.x;
-                        cy = loy = hiy = p.y;
-                        cz = loz = hiz = p.z;
-                        ro = 0.0f;
-                        pointlike = true;
-                    } else {
-                        cx = S[s].a.x; cy = S[s].a.y; cz = S[s].a.z; ro = S[s].a.w;
-                        lox = S[s].b.x; loy = S[s].b.y; loz = S[s].b.z;
-                        hix = S[s].c.x; hiy = S[s].c.y; hiz = S[s].c.z;
-                        pointlike = S[s].d.w == 1;
-                        sleaf[s] = S[s].d.x < 0;  // a leaf (bucket) has no children
-                        c0[s] = S[s].d.x;
-                        c1[s] = S[s].d.y;
-                        sfirst[s] = S[s].d.z;
-                        nsrc_cell[s] = S[s].d.w;
-                        nadd[s] = sleaf[s] ? S[s].d.w : 2;
-                    }
-                    d2 = d2_ordered(__fsub_rn(K.a.x, cx), __fsub_rn(K.a.y, cy), __fsub_rn(K.a.z, cz));
-                    const float thr = __fadd_rn(__fmul_rn(1.5f, rk), ro);
-                    const float gx = gap_axis(lox, hix, K.b.x, K.c.x);
-                    const float gy = gap_axis(loy, hiy, K.b.y, K.c.y);
-                    const float gz = gap_axis(loz, hiz, K.b.z, K.c.z);
-                    const float gap2 = d2_ordered(gx, gy, gz);
-                    acc = d2 > __fmul_rn(thr, thr) && gap2 >= four_eps2;
-                    if (MODE != 0 && !pointlike) {
+                bool acc = false, ptl = false, mid = false, pp = false, open = false, need = false;
+                int4 sd = make_int4(-1, -1, 0, 0);
+                if (valid) {
+                    const WalkNode S = walk_source<PER>(w, e, q0, ib);
+                    const float ro = S.a.w;
+                    sd = S.d;
+                    ptl = sd.w == 1;
+                    const float d2 = d2_ordered(__fsub_rn(K.a.x, S.a.x), __fsub_rn(K.a.y, S.a.y), __fsub_rn(K.a.z, S.a.z));
+                    const float thr = __fadd_rn(rk15, ro);
+                    const float gap2 = d2_ordered(gap_axis(S.b.x, S.c.x, K.b.x, K.c.x),
+                                                  gap_axis(S.b.y, S.c.y, K.b.y, K.c.y),
+                                                  gap_axis(S.b.z, S.c.z, K.b.z, K.c.z));
+                    acc = d2 > __fmul_rn(thr, thr) && gap2 >= w.four_eps2;
+                    if (MODE != 0 && !ptl) {
                         float te;
-                        int band = mlp_band(K, S[s], d2, gap2, four_eps2, band_lo, band_hi, te);
+                        int band = mlp_band(K, S, d2, gap2, w.four_eps2, w.band_lo, w.band_hi, te);
                         if (MODE == 1) {
                             if (band == 3 && decided) {
                                 band = decided == WALK_NET_ACC ? 1 : 2;  // the network has decided
                             } else if (band == 3 && !(ak > 0.0f)) {
                                 band = acc ? 1 : 2;  // no acceleration estimate: the fixed criterion decides
                             } else if (band == 3) {
-                                mlp_pair_features(K, S[s], mnorm[entry_index(e[s], ib)], ak, eps, f);
-                                band = mlp_surrogate(reinterpret_cast<const float*>(walk_smem + MLPP_SUR), f, te, tau,
-                                                     margin);
+                                float f[MLP_F];
+                                mlp_pair_features(K, S, w.mnorm[entry_index(e, ib)], ak, w.eps, f);
+                                band = mlp_surrogate(reinterpret_cast<const float*>(walk_smem + MLPP_SUR), f, te, w.tau,
+                                                     w.margin);
                             }
                             acc = band == 1;
                             need = band == 3;
                         } else if (band == 3) {
                             const unsigned long long q = atomicAdd(&ctr->n_audit, 1ull);
-                            if ((long long)q < audit_cap) audit_pairs[q] = make_int2(k, (int)e[s]);
+                            if ((long long)q < w.audit_cap) w.audit_pairs[q] = make_int2(k, (int)e);
+                        }
+                    }
+                    // a pair for the network gives no output until it has been decided
+                    if (MODE == 1 && need) {
+                        valid = false;
+                    } else if (!acc) {
+                        if (!kg) {
+                            mid = ptl || ro <= rk;  // defer
+                            open = !mid;
+                        } else if (ptl) {
+                            pp = true;
+                        } else {
+                            const float u = __fadd_rn(ro, bk);
+                            mid = d2 > __fmul_rn(u, u);  // PC
+                            pp = !mid && sd.x < 0;       // a leaf (bucket) has no children
+                            open = !mid && !pp;
                         }
                     }
                 }
-                if (MODE == 1) {
-                    // a pair for the network waits in the buffer and gives no output this step
-                    const unsigned int nm = __ballot_sync(FMM_FULL_MASK, need);
-                    if (need) {
-                        const int slot = npend + __popc(nm & lt);
-                        pend_e[slot] = e[s];
+                // this warp's outcomes, in queue order
+                const bool leaf = sd.x < 0;
+                const unsigned int mA = __ballot_sync(FMM_FULL_MASK, acc && !ptl);
+                const unsigned int mAp = __ballot_sync(FMM_FULL_MASK, acc && ptl);
+                const unsigned int mX = __ballot_sync(FMM_FULL_MASK, mid);
+                // a group opens no leaf; any other sink has no PP entries
+                const unsigned int mP = __ballot_sync(FMM_FULL_MASK, kg ? pp : (open && leaf));
+                const unsigned int mO = __ballot_sync(FMM_FULL_MASK, open && !leaf);
+                const unsigned int mW = MODE == 1 ? __ballot_sync(FMM_FULL_MASK, need) : 0u;
+                int qat = 2 * __popc(mO & lt), qtot = 2 * __popc(mO);
+                if (!kg && mP) {
+                    // leaves add 1 to 16 entries each: their counts bit by bit
+                    const unsigned int c = open && leaf ? (unsigned int)sd.w : 0u;
 #pragma unroll
-                        for (int q = 0; q < MLP_F; q++) pend_f[slot * MLP_F + q] = f[q];
-                    }
-                    npend += __popc(nm);
-                    if (need) {
-                        valid[s] = false;
-                        nadd[s] = 0;
+                    for (int b = 0; b < 5; b++) {
+                        const unsigned int m = __ballot_sync(FMM_FULL_MASK, (c >> b) & 1u);
+                        qat += __popc(m & lt) << b;
+                        qtot += __popc(m) << b;
                     }
                 }
-                ptl[s] = pointlike;
-                if (valid[s]) {
-                    if (acc) {
-                        out[s] = OUT_ACCEPT;
-                    } else if (!kg) {
-                        out[s] = (pointlike || ro <= rk) ? OUT_DEFER : OUT_OPEN;
-                    } else if (pointlike) {
-                        out[s] = OUT_PP;
-                    } else {
-                        const float u = __fadd_rn(ro, bk);
-                        if (d2 > __fmul_rn(u, u)) out[s] = OUT_PC;
-                        else out[s] = sleaf[s] ? OUT_PP : OUT_OPEN;
+                int oA = na + __popc(mA & lt), oAp = nap + __popc(mAp & lt), oX = nx + __popc(mX & lt),
+                    oP = npp + __popc(mP & lt), oW = MODE == 1 ? nw + __popc(mW & lt) : 0;
+                qat += total - ncl;
+                int tA = __popc(mA), tAp = __popc(mAp), tX = __popc(mX), tP = kg ? __popc(mP) : 0,
+                    tW = MODE == 1 ? __popc(mW) : 0, tQ = qtot;
+                if (TEAM > 1) {
+                    // the counts of the team's warps: four of 8 bits (at most 32 * TEAM = 128 each), then
+                    // the network's of 8 bits and the queue's (at most 512 * TEAM)
+                    static_assert(WIN <= 255, "packed step counts");
+                    if (lane == 0)
+                        sh.cnt[par][wl] = make_uint2((unsigned)tA | (unsigned)tAp << 8 | (unsigned)tX << 16 | (unsigned)tP << 24,
+                                                     (unsigned)tQ | (unsigned)tW << 24);
+                    __syncthreads();
+                    uint2 before = make_uint2(0u, 0u), all = make_uint2(0u, 0u);
+#pragma unroll
+                    for (int v = 0; v < TEAM; v++) {
+                        const uint2 c = sh.cnt[par][v];
+                        if (v == tw) before = all;
+                        all.x += c.x;
+                        all.y += c.y;
                     }
-                    if (out[s] != OUT_OPEN) nadd[s] = 0;
+                    oA += before.x & 255u;
+                    oAp += (before.x >> 8) & 255u;
+                    oX += (before.x >> 16) & 255u;
+                    oP += before.x >> 24;
+                    qat += before.y & 0xffffffu;
+                    tA = all.x & 255u;
+                    tAp = (all.x >> 8) & 255u;
+                    tX = (all.x >> 16) & 255u;
+                    tP = all.x >> 24;
+                    tQ = all.y & 0xffffffu;
+                    if (MODE == 1) {
+                        oW += before.y >> 24;
+                        tW = all.y >> 24;
+                    }
+                    par ^= 1;
                 }
+                if (na + nap + tA + tAp > cap || nx + tX > cap || npp + tP > cap || total - ncl + tQ > cap ||
+                    (MODE == 1 && nw + tW > cap)) {
+                    overflow = true;
+                    break;
+                }
+                if (acc) {
+                    if (ptl) A[cap - 1 - oAp] = e;
+                    else A[oA] = e;
+                }
+                if (mid) X[oX] = e;
+                if (pp) {
+                    P[oP] = e;
+                    srcpp += sd.w;
+                }
+                if (MODE == 1 && need) W[oW] = e;
+                // the children of opened cells, and the particles of opened leaves, stay in the source's copy
+                const unsigned int qb = PER ? entry_copy(e, ib) << ib : 0u;
+                if (open && !leaf) {
+                    Q[qat] = (unsigned int)sd.x | qb;
+                    Q[qat + 1] = (unsigned int)sd.y | qb;
+                }
+                if (!kg) {
+                    // one opened leaf at a time, its particles along the lanes
+                    for (unsigned int m = mP; m; m &= m - 1) {
+                        const int src = __ffs(m) - 1;
+                        const int at = __shfl_sync(FMM_FULL_MASK, qat, src), n = __shfl_sync(FMM_FULL_MASK, sd.w, src);
+                        const unsigned int v = __shfl_sync(FMM_FULL_MASK, (unsigned int)sd.z | qb, src);
+                        if (lane < n) Q[at + lane] = (v + (unsigned int)lane) | FMM_PARTICLE_BIT;
+                    }
+                }
+                const int seen = total;
+                na += tA;
+                nap += tAp;
+                nx += tX;
+                npp += tP;
+                nw += tW;
+                total += tQ;
+                // the next step's entries must be in place: a team's barrier is needed only when it reads
+                // what this step appended (what earlier steps appended lies behind this step's barrier)
+                if (TEAM == 1 || min(base + WIN, total) > seen) team_sync<TEAM>();
             }
-            // ranks in queue order: slot by slot, lanes in order within a slot
-            unsigned int mA[E], mAp[E], mD[E], mC[E], mP[E];
-            int incl[E], tot[E];
-            long long tA = 0, tAp = 0, tD = 0, tC = 0, tP = 0, tQ = 0;
-#pragma unroll
-            for (int s = 0; s < E; s++) {
-                mA[s] = mAp[s] = mD[s] = mC[s] = mP[s] = 0u;
-                incl[s] = tot[s] = 0;
-                if (s >= ns) continue;
-                mA[s] = __ballot_sync(FMM_FULL_MASK, out[s] == OUT_ACCEPT && !ptl[s]);
-                mAp[s] = __ballot_sync(FMM_FULL_MASK, out[s] == OUT_ACCEPT && ptl[s]);
-                mD[s] = __ballot_sync(FMM_FULL_MASK, out[s] == OUT_DEFER);
-                mC[s] = __ballot_sync(FMM_FULL_MASK, out[s] == OUT_PC);
-                mP[s] = __ballot_sync(FMM_FULL_MASK, out[s] == OUT_PP);
-                int v = nadd[s];
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_up_sync(FMM_FULL_MASK, v, o);
-                    if (lane >= o) v += t;
-                }
-                incl[s] = v;
-                tot[s] = __shfl_sync(FMM_FULL_MASK, v, 31);
-                tA += __popc(mA[s]);
-                tAp += __popc(mAp[s]);
-                tD += __popc(mD[s]);
-                tC += __popc(mC[s]);
-                tP += __popc(mP[s]);
-                tQ += tot[s];
-            }
-            if (na + nap + tA + tAp > cap_scr || nd + tD > cap_scr || npc + tC > cap_scr || npp + tP > cap_scr ||
-                nq + tQ > cap_scr) {
+            if (MODE == 0 || MODE == 2 || overflow || nw == 0) break;
+            // the queue is dry: the network decides the waiting pairs, 32 per warp and turn
+            if (total - ncl + nw > cap) {
                 overflow = true;
                 break;
             }
+            team_sync<TEAM>();
+            for (int b = tw * 32; b < nw; b += WIN) {
+                const int cnt = min(32, nw - b);
+                float f[MLP_F];
 #pragma unroll
-            for (int s = 0; s < E; s++) {
-                if (s >= ns) continue;
-                if (out[s] == OUT_ACCEPT) {
-                    if (ptl[s]) A[cap_scr - 1 - (nap + __popc(mAp[s] & lt))] = e[s];
-                    else A[na + __popc(mA[s] & lt)] = e[s];
+                for (int q = 0; q < MLP_F; q++) f[q] = 0.0f;
+                unsigned int pe = 0u;
+                if (lane < cnt) {
+                    pe = W[b + lane];
+                    const unsigned int j = entry_index(pe, ib);
+                    mlp_pair_features(K, w.node[j], w.mnorm[j], ak, w.eps, f);
                 }
-                if (out[s] == OUT_DEFER) D[nd + __popc(mD[s] & lt)] = e[s];
-                if (out[s] == OUT_PC) C[npc + __popc(mC[s] & lt)] = e[s];
-                if (out[s] == OUT_PP) {
-                    P[npp + __popc(mP[s] & lt)] = e[s];
-                    srcpp += (e[s] & FMM_PARTICLE_BIT) ? 1 : nsrc_cell[s];
-                }
-                if (out[s] == OUT_OPEN) {
-                    // the children, or a leaf's particles, stay in the source's copy
-                    const long long pos = nq + incl[s] - nadd[s];
-                    const unsigned int qb = PER ? entry_copy(e[s], ib) << ib : 0u;
-                    if (sleaf[s]) {
-                        for (int j = 0; j < nadd[s]; j++)
-                            Q[pos + j] = ((unsigned int)(sfirst[s] + j) | qb) | FMM_PARTICLE_BIT;
-                    } else {
-                        Q[pos] = (unsigned int)c0[s] | qb;
-                        Q[pos + 1] = (unsigned int)c1[s] | qb;
-                    }
-                }
-                na += __popc(mA[s]);
-                nap += __popc(mAp[s]);
-                nd += __popc(mD[s]);
-                npc += __popc(mC[s]);
-                npp += __popc(mP[s]);
-                nq += tot[s];
+                const float pred = mlp_predict_warp(walk_smem, mlp_scratch, f, lane,
+                                                    cnt == 32 ? FMM_FULL_MASK : (1u << cnt) - 1u);
+                if (lane < cnt) Q[total - ncl + b + lane] = pe | (pred < w.tau ? WALK_NET_ACC : WALK_NET_REJ);
             }
-            __syncwarp();
-            if (MODE == 1) {
-                // evaluate 32 waiting pairs (or the rest once the queue is dry) and return them
-                // to the queue with their decisions
-                while (npend >= 32 || (npend > 0 && base >= ncl + nq)) {
-                    const int cnt = npend < 32 ? npend : 32;
-                    if (nq + cnt > cap_scr) {
-                        overflow = true;
-                        break;
-                    }
-                    float f[MLP_F];
-                    const bool have = lane < cnt;
-#pragma unroll
-                    for (int q = 0; q < MLP_F; q++) f[q] = have ? pend_f[lane * MLP_F + q] : 0.0f;
-                    const unsigned int pe = have ? pend_e[lane] : 0u;
-                    const float pred = mlp_predict_warp(walk_smem, mlp_scratch, f, lane,
-                                                        cnt == 32 ? FMM_FULL_MASK : (1u << cnt) - 1u);
-                    if (have) Q[nq + lane] = pe | (pred < tau ? WALK_NET_ACC : WALK_NET_REJ);
-                    n_mlp += cnt;
-                    nq += cnt;
-                    // move the rest (fewer than 32) to the front of the buffer
-                    const int rest = npend - cnt;
-                    unsigned int me = 0u;
-                    float mf[MLP_F];
-                    if (lane < rest) {
-                        me = pend_e[cnt + lane];
-#pragma unroll
-                        for (int q = 0; q < MLP_F; q++) mf[q] = pend_f[(cnt + lane) * MLP_F + q];
-                    }
-                    __syncwarp();
-                    if (lane < rest) {
-                        pend_e[lane] = me;
-#pragma unroll
-                        for (int q = 0; q < MLP_F; q++) pend_f[lane * MLP_F + q] = mf[q];
-                    }
-                    npend = rest;
-                    __syncwarp();
-                }
-                if (overflow) break;
-            }
+            base = total;
+            total += nw;
+            n_mlp += (unsigned long long)nw;
+            nw = 0;
+            team_sync<TEAM>();
         }
         if (overflow) {
-            if (lane == 0) atomicOr(&ctr->overflow, 1u);
+            if (tl == 0) atomicOr(&ctr->overflow, 1u);
             continue;
         }
-        w_entries += (unsigned long long)(ncl + nq);
-        w_max = max(w_max, (unsigned long long)(ncl + nq));
-        // local-expansion entries of this sink: multipole sources (M2L) and point sources (P2L) in
-        // two lists, each in queue order
-        unsigned long long off = 0, offp = 0;
-        if (lane == 0) {
-            if (na) {
-                off = atomicAdd(&ctr->cc_len, (unsigned long long)na);
-                atomicAdd(&ctr->lv_cc[level], (unsigned long long)na);
-            }
-            if (nap) {
-                offp = atomicAdd(&ctr->cp_len, (unsigned long long)nap);
-                atomicAdd(&ctr->lv_cp[level], (unsigned long long)nap);
-            }
+        w_entries += (unsigned long long)total;
+        w_max = max(w_max, total);
+        // Room in the sink's lists: multipole sources (M2L) and point sources (P2L), and a group's PP and
+        // PC entries or any other sink's checklist for its children, each in queue order.  One lane per
+        // counter, so the atomics are in flight together.
+        if (TEAM > 1 && kg) {
+            srcpp = (int)__reduce_add_sync(FMM_FULL_MASK, (unsigned int)srcpp);
+            if (lane == 0 && srcpp) atomicAdd(&sh.srcpp, (unsigned int)srcpp);
         }
-        off = __shfl_sync(FMM_FULL_MASK, off, 0);
-        offp = __shfl_sync(FMM_FULL_MASK, offp, 0);
-        if ((long long)(off + na) > cap_cc || (long long)(offp + nap) > cap_cp) {
-            if (lane == 0) atomicOr(&ctr->overflow, 1u);
+        unsigned long long at = 0;
+        if (tl < 5) {
+            unsigned long long* c = tl == 0   ? &ctr->cc_len
+                                    : tl == 1 ? &ctr->cp_len
+                                    : tl == 2 ? (kg ? &ctr->pp_len : &ctr->lv_cl[w.level + 1])
+                                    : tl == 3 ? &ctr->pc_len
+                                              : &ctr->n_groups;
+            const unsigned long long v = tl == 0 ? na : tl == 1 ? nap : tl == 2 ? (kg ? npp : nx) : tl == 3 ? nx : 1;
+            if ((kg || tl < 3) && v) at = atomicAdd(c, v);
+            if (TEAM > 1) sh.at[tl] = at;
+        } else if (tl < 7) {  // the level's own counts
+            const unsigned long long v = tl == 5 ? na : nap;
+            if (v) atomicAdd(tl == 5 ? &ctr->lv_cc[w.level] : &ctr->lv_cp[w.level], v);
+        }
+        unsigned long long off, offp, xo, co, gi;
+        if (TEAM == 1) {
+            off = __shfl_sync(FMM_FULL_MASK, at, 0);
+            offp = __shfl_sync(FMM_FULL_MASK, at, 1);
+            xo = __shfl_sync(FMM_FULL_MASK, at, 2);
+            co = __shfl_sync(FMM_FULL_MASK, at, 3);
+            gi = __shfl_sync(FMM_FULL_MASK, at, 4);
+        } else {
+            __syncthreads();
+            off = sh.at[0];
+            offp = sh.at[1];
+            xo = sh.at[2];
+            co = sh.at[3];
+            gi = sh.at[4];
+        }
+        bool fits = (long long)(off + na) <= w.cap_cc && (long long)(offp + nap) <= w.cap_cp;
+        if (kg) fits = fits && (long long)(xo + npp) <= w.cap_pp && (long long)(co + nx) <= w.cap_pc && (long long)gi < w.cap_groups;
+        else fits = fits && (long long)(xo + nx) <= w.cap_cl;
+        if (!fits) {
+            if (tl == 0) atomicOr(&ctr->overflow, 1u);
             continue;
         }
-        for (long long i = lane; i < na; i += 32) {
-            cc[off + i] = A[i];
-            cc_sink[off + i] = k;
+        for (int i = tl; i < na; i += WIN) {
+            w.cc[off + i] = A[i];
+            w.cc_sink[off + i] = k;
         }
-        for (long long i = lane; i < nap; i += 32) {
-            cp[offp + i] = A[cap_scr - 1 - i];
-            cp_sink[offp + i] = k;
+        for (int i = tl; i < nap; i += WIN) {
+            w.cp[offp + i] = A[cap - 1 - i];
+            w.cp_sink[offp + i] = k;
         }
-        if (lane == 0) {
-            lcc_off[k] = off;
-            lcc_len[k] = (int)na;
-            lcp_off[k] = offp;
-            lcp_len[k] = (int)nap;
+        if (tl == 0) {
+            w.lcc_off[k] = off;
+            w.lcc_len[k] = na;
+            w.lcp_off[k] = offp;
+            w.lcp_len[k] = nap;
         }
         if (kg) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) srcpp += __shfl_xor_sync(FMM_FULL_MASK, srcpp, o);
-            unsigned long long po = 0, co = 0, gi = 0;
-            if (lane == 0) {
-                po = atomicAdd(&ctr->pp_len, (unsigned long long)npp);
-                co = atomicAdd(&ctr->pc_len, (unsigned long long)npc);
-                gi = atomicAdd(&ctr->n_groups, 1ull);
-            }
-            po = __shfl_sync(FMM_FULL_MASK, po, 0);
-            co = __shfl_sync(FMM_FULL_MASK, co, 0);
-            gi = __shfl_sync(FMM_FULL_MASK, gi, 0);
-            if ((long long)(po + npp) > cap_pp || (long long)(co + npc) > cap_pc || (long long)gi >= cap_groups) {
-                if (lane == 0) atomicOr(&ctr->overflow, 1u);
-                continue;
-            }
-            for (long long i = lane; i < npp; i += 32) pp[po + i] = P[i];
-            for (long long i = lane; i < npc; i += 32) pc[co + i] = C[i];
-            if (lane == 0) {
+            if (TEAM == 1) srcpp = (int)__reduce_add_sync(FMM_FULL_MASK, (unsigned int)srcpp);
+            else srcpp = (int)sh.srcpp;
+            for (int i = tl; i < npp; i += WIN) w.pp[xo + i] = P[i];
+            for (int i = tl; i < nx; i += WIN) w.pc[co + i] = C[i];
+            if (tl == 0) {
                 Group g;
                 g.cell = k;
                 g.first = K.d.z;
                 g.count = K.d.w;
                 g.pp_src = srcpp;
-                g.pp_off = po;
+                g.pp_off = xo;
                 g.pc_off = co;
-                g.pp_len = (int)npp;
-                g.pc_len = (int)npc;
-                groups[gi] = g;
+                g.pp_len = npp;
+                g.pc_len = nx;
+                w.groups[gi] = g;
             }
         } else {
-            unsigned long long doff = 0;
-            if (lane == 0) doff = atomicAdd(&ctr->lv_cl[level + 1], (unsigned long long)nd);
-            doff = __shfl_sync(FMM_FULL_MASK, doff, 0);
-            if ((long long)(doff + nd) > cap_cl) {
-                if (lane == 0) atomicOr(&ctr->overflow, 1u);
-                continue;
-            }
-            for (long long i = lane; i < nd; i += 32) cl_next[doff + i] = D[i];
-            if (lane < 2) {
-                int c = lane == 0 ? K.d.x : K.d.y;
-                if (cnact[c] > 0) {
-                    unsigned long long fj = atomicAdd(&ctr->lv_front[level + 1], 1ull);
-                    if ((long long)fj < cap_front) {
-                        f_cell_next[fj] = c;
-                        f_cloff_next[fj] = doff;
-                        f_cllen_next[fj] = (int)nd;
+            for (int i = tl; i < nx; i += WIN) w.cl_next[xo + i] = D[i];
+            if (tl < 2) {
+                const int c = tl == 0 ? K.d.x : K.d.y;
+                if (w.cnact[c] > 0) {
+                    const unsigned long long fj = atomicAdd(&ctr->lv_front[w.level + 1], 1ull);
+                    if ((long long)fj < w.cap_front) {
+                        w.f_cell_next[fj] = c;
+                        w.f_cloff_next[fj] = xo;
+                        w.f_cllen_next[fj] = nx;
                     } else {
                         atomicOr(&ctr->overflow, 1u);
                     }
@@ -511,11 +528,34 @@ __global__ void __launch_bounds__(WALK_THREADS, MODE == 1 ? 4 : FMM_WALK_MINB) k
             }
         }
     }
-    if (MODE == 1 && lane == 0 && n_mlp) atomicAdd(&ctr->n_mlp, n_mlp);
-    if (lane == 0 && w_entries) {
-        atomicAdd(&ctr->lv_entries[level], w_entries);
-        atomicMax(&ctr->lv_max_entries[level], w_max);
+    if (tl == 0) {
+        if (MODE == 1 && n_mlp) atomicAdd(&ctr->n_mlp, n_mlp);
+        if (w_entries) {
+            atomicAdd(&ctr->lv_entries[w.level], w_entries);
+            atomicMax(&ctr->lv_max_entries[w.level], (unsigned long long)w_max);
+        }
     }
+}
+
+template <int MODE, bool PER>
+__global__ void __launch_bounds__(WALK_THREADS, MODE == 1 ? 4 : FMM_WALK_MINB) k_walk_level(const __grid_constant__ WalkIO w)
+{
+    __shared__ WalkShared sh;
+    extern __shared__ __align__(16) unsigned char walk_smem[];
+    DevCounters* const ctr = w.ctr;
+    const unsigned long long n_front = *(volatile unsigned long long*)&ctr->lv_front[w.level];
+    // this level's sinks go to the walked-cell list after the levels before it
+    const unsigned long long wbase = *(volatile unsigned long long*)&ctr->lv_base[w.level];
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctr->lv_base[w.level + 1] = wbase + n_front;
+    const bool team = n_front < (unsigned long long)gridDim.x * FMM_WALK_TEAM_SINKS;
+    if ((unsigned long long)blockIdx.x * (team ? 1 : WALK_WPB) >= n_front) return;  // no sink is left for this block
+    if (MODE == 1) {
+        mlp_load_smem(w.mlp_packed, walk_smem);
+        __syncthreads();
+    }
+    unsigned char* mlp_scratch = walk_smem + MLPP_SIZE + (threadIdx.x >> 5) * MLP_WARP_SCRATCH;
+    if (team) walk_sinks<MODE, PER, WALK_WPB>(w, n_front, wbase, sh, walk_smem, mlp_scratch);
+    else walk_sinks<MODE, PER, 1>(w, n_front, wbase, sh, walk_smem, mlp_scratch);
 }
 
 #define LOCAL_WPB 2
@@ -832,30 +872,72 @@ int fmm_walk_warps(int device)
 cudaError_t fmm_launch_walk_level(DevTree& t, DevWalk& w, DevCounters* ctr, const WalkArgs& a, cudaStream_t s)
 {
     const int cur = a.level_parity, nxt = cur ^ 1;
-    // persistent grid: every warp owns a scratch slot; idle warps exit after one atomic
+    // persistent grid: every warp owns a scratch slot; blocks without a sink exit at once
     const int blocks = w.n_warps / WALK_WPB;
-#define WALK_ARGS                                                                                                   \
-    t.node, t.posf, t.cnact, w.f_cell[cur], w.f_cloff[cur], w.f_cllen[cur], a.level, w.cl[cur], w.f_cell[nxt],      \
-        w.f_cloff[nxt], w.f_cllen[nxt], w.cap_front, w.cl[nxt], w.cap_cl, w.lcc_off, w.lcc_len, w.lcp_off,          \
-        w.lcp_len, w.wcells, w.pp, w.cap_pp, w.pc, w.cap_pc, w.cc, w.cc_sink, w.cap_cc, w.cp, w.cp_sink, w.cap_cp, w.groups, w.cap_groups, w.scratch, w.cap_scratch, ctr, \
-        a.bucket, a.group, a.four_eps2, t.mnorm, t.amin, a.eps, a.band_lo, a.band_hi, a.tau, a.margin, a.mlp_packed, a.audit_pairs, \
-        a.audit_cap, t.graded ? t.nogroup : nullptr, periodic_args(t)
+    WalkIO io;
+    io.node = t.node;
+    io.posf = t.posf;
+    io.cnact = t.cnact;
+    io.f_cell = w.f_cell[cur];
+    io.f_cloff = w.f_cloff[cur];
+    io.f_cllen = w.f_cllen[cur];
+    io.cl_cur = w.cl[cur];
+    io.f_cell_next = w.f_cell[nxt];
+    io.f_cloff_next = w.f_cloff[nxt];
+    io.f_cllen_next = w.f_cllen[nxt];
+    io.cl_next = w.cl[nxt];
+    io.lcc_off = w.lcc_off;
+    io.lcp_off = w.lcp_off;
+    io.lcc_len = w.lcc_len;
+    io.lcp_len = w.lcp_len;
+    io.wcells = w.wcells;
+    io.pp = w.pp;
+    io.pc = w.pc;
+    io.cc = w.cc;
+    io.cp = w.cp;
+    io.cc_sink = w.cc_sink;
+    io.cp_sink = w.cp_sink;
+    io.groups = w.groups;
+    io.scratch = w.scratch;
+    io.ctr = ctr;
+    io.cap_front = w.cap_front;
+    io.cap_cl = w.cap_cl;
+    io.cap_pp = w.cap_pp;
+    io.cap_pc = w.cap_pc;
+    io.cap_cc = w.cap_cc;
+    io.cap_cp = w.cap_cp;
+    io.cap_groups = w.cap_groups;
+    io.cap_scr = w.cap_scratch;
+    io.level = a.level;
+    io.group = a.group;
+    io.four_eps2 = a.four_eps2;
+    io.mnorm = t.mnorm;
+    io.amin = t.amin;
+    io.eps = a.eps;
+    io.band_lo = a.band_lo;
+    io.band_hi = a.band_hi;
+    io.tau = a.tau;
+    io.margin = a.margin;
+    io.mlp_packed = a.mlp_packed;
+    io.audit_pairs = a.audit_pairs;
+    io.audit_cap = a.audit_cap;
+    io.nogroup = t.graded ? t.nogroup : nullptr;
+    io.pa = periodic_args(t);
     // the learned and audit walks take isolated boxes only (the host refuses the combinations)
     if (a.mode != 0 && t.per_R > 0) return cudaErrorInvalidValue;
     if (a.mode == 1) {
-        const size_t smem = MLPP_SIZE + (size_t)WALK_WPB * (MLP_WARP_SCRATCH + WALK_PEND_BYTES);
+        const size_t smem = MLPP_SIZE + (size_t)WALK_WPB * MLP_WARP_SCRATCH;
         static std::atomic<unsigned long long> attr{0};
         cudaError_t e = fmm_smem_attr_once(k_walk_level<1, false>, (int)smem, attr);
         if (e != cudaSuccess) return e;
-        k_walk_level<1, false><<<blocks, WALK_THREADS, smem, s>>>(WALK_ARGS);
+        k_walk_level<1, false><<<blocks, WALK_THREADS, smem, s>>>(io);
     } else if (a.mode == 2) {
-        k_walk_level<2, false><<<blocks, WALK_THREADS, 0, s>>>(WALK_ARGS);
+        k_walk_level<2, false><<<blocks, WALK_THREADS, 0, s>>>(io);
     } else if (t.per_R > 0) {
-        k_walk_level<0, true><<<blocks, WALK_THREADS, 0, s>>>(WALK_ARGS);
+        k_walk_level<0, true><<<blocks, WALK_THREADS, 0, s>>>(io);
     } else {
-        k_walk_level<0, false><<<blocks, WALK_THREADS, 0, s>>>(WALK_ARGS);
+        k_walk_level<0, false><<<blocks, WALK_THREADS, 0, s>>>(io);
     }
-#undef WALK_ARGS
     return cudaGetLastError();
 }
 
