@@ -18,9 +18,9 @@
 #include "f64bits.cuh"
 #include "fmm_internal.cuh"
 
-__device__ __forceinline__ int target_rung(float ax, float ay, float az, double eps, double dt0, int R)
+// The target rung in FP64: the definition.
+__device__ __noinline__ int target_rung_f64(float ax, float ay, float az, double eps, double dt0, int R)
 {
-    if (R == 0) return 0;  // a single rung: nothing to decide (and FP64 sqrt and division are slow here)
     double x = ax, y = ay, z = az;
     double a2 = __dadd_rn(__dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y)), __dmul_rn(z, z));
     double am = __dsqrt_rn(a2);
@@ -31,12 +31,46 @@ __device__ __forceinline__ int target_rung(float ax, float ay, float az, double 
     return r;
 }
 
+// The same rung, decided in FP32 where FP32 can decide it.  dt0 <= Delta T 2^r is
+// |a|^2 <= t0 16^r with t0 = (0.04 eps / dt0^2)^2 (t0 = 0: outside FP32's range, never decided here).
+// The FP32 square is within 3e-7 of the exact one (three squares and two sums, each rounded once;
+// the range below keeps lost subnormals far under that), t0's rounding within 6e-8 and the FP64
+// definition's own roundings within 1e-14, so a square further than 1e-6 from the thresholds on both
+// sides of it has the definition's rung; the others (one particle in about a million) take it.  The
+// FP64 square roots and division (FP64 issues at 1/64 of the FP32 rate, and a warp pays in full for one
+// active lane) made the kick-drift of a 256^3 box with a tenth active 1.62 ms, 0.8 TB/s; it takes
+// 0.46 ms, 2.8 TB/s, this way, bound by the FP64 multiply-adds of the kicks and the drift.
+__device__ __forceinline__ int target_rung(float ax, float ay, float az, double eps, double dt0, int R, float t0)
+{
+    if (R == 0) return 0;  // a single rung: nothing to decide
+    const float a2 = __fmaf_rn(ax, ax, __fmaf_rn(ay, ay, __fmul_rn(az, az)));
+    if (a2 == 0.0f && ax == 0.0f && ay == 0.0f && az == 0.0f) return 0;
+    if (t0 > 0.0f && a2 > 1e-30f && a2 < 1e37f) {
+        int r = 0;
+        float t = t0;
+        while (r < R && a2 > t) {
+            r++;
+            t *= 16.0f;
+        }
+        const bool above = r == 0 || a2 > 0.0625f * t * 1.000001f, below = r == R || a2 < t * 0.999999f;
+        if (above && below) return r;
+    }
+    return target_rung_f64(ax, ay, az, eps, dt0, R);
+}
+
+// t0 of target_rung; 0 where it or its first multiples leave FP32's normal range
+static float rung_threshold(double eps, double dt0)
+{
+    const double q = 0.04 * eps / (dt0 * dt0), t = q * q;
+    return t > 1e-36 && t < 1e36 ? (float)t : 0.0f;
+}
+
 __global__ void k_assign_rungs(const float* __restrict__ acc, unsigned char* __restrict__ rung, long long n,
-                               double eps, double dt0, int R)
+                               double eps, double dt0, int R, float t0)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    rung[i] = (unsigned char)target_rung(acc[i], acc[n + i], acc[2 * n + i], eps, dt0, R);
+    rung[i] = (unsigned char)target_rung(acc[i], acc[n + i], acc[2 * n + i], eps, dt0, R, t0);
 }
 
 // dt0 2^-k as ldexp gives it, by one exact multiplication with the power of two built from its bits
@@ -50,7 +84,8 @@ __device__ __forceinline__ double pow2_scale(double dt0, int k)
 // (f64bits.cuh) and give the same values.
 __global__ void k_kick_drift(double* __restrict__ pos, double* __restrict__ vel, const float* __restrict__ acc,
                              unsigned char* __restrict__ rung, unsigned char* __restrict__ active_next, long long n,
-                             double eps, double dt0, int R, long long s, int closing, unsigned int* __restrict__ status)
+                             double eps, double dt0, int R, float t0, long long s, int closing,
+                             unsigned int* __restrict__ status)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -65,7 +100,7 @@ __global__ void k_kick_drift(double* __restrict__ pos, double* __restrict__ vel,
             vy += ay * hk;
             vz += az * hk;
         }
-        int rt = target_rung(fx, fy, fz, eps, dt0, R);
+        int rt = target_rung(fx, fy, fz, eps, dt0, R, t0);
         int rn = rt;
         if (rt < r) {
             rn = rt;
@@ -96,7 +131,7 @@ cudaError_t fmm_launch_kick_drift(double* pos, double* vel, const float* acc, un
                                   int substep, int closing, DevCounters* ctr, cudaStream_t s)
 {
     k_kick_drift<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(pos, vel, acc, rung, active_next, n, eps, dt0,
-                                                                max_rung, substep, closing, &ctr->status);
+                                                                max_rung, rung_threshold(eps, dt0), substep, closing, &ctr->status);
     return cudaGetLastError();
 }
 
@@ -110,7 +145,7 @@ cudaError_t fmm_launch_kick_drift(double* pos, double* vel, const float* acc, un
 __global__ void k_kick_drift_i32(unsigned int* __restrict__ ipos, float* __restrict__ vel,
                                  const float* __restrict__ acc, unsigned char* __restrict__ rung,
                                  unsigned char* __restrict__ active_next, long long n, double eps, double dt0, int R,
-                                 long long s, int closing, int periodic, unsigned int* __restrict__ status)
+                                 float t0, long long s, int closing, int periodic, unsigned int* __restrict__ status)
 {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -118,12 +153,12 @@ __global__ void k_kick_drift_i32(unsigned int* __restrict__ ipos, float* __restr
     float v32[3] = {vel[i], vel[n + i], vel[2 * n + i]};
     if ((s & ((1LL << (R - r)) - 1)) == 0) {
         const float f[3] = {acc[i], acc[n + i], acc[2 * n + i]};
-        double v[3] = {v32[0], v32[1], v32[2]};
+        double v[3] = {fmm_f2d(v32[0]), fmm_f2d(v32[1]), fmm_f2d(v32[2])};
         if (closing) {
-            const double hk = ldexp(dt0, -r - 1);
-            for (int a = 0; a < 3; a++) v[a] = __dadd_rn(v[a], __dmul_rn((double)f[a], hk));
+            const double hk = pow2_scale(dt0, r + 1);
+            for (int a = 0; a < 3; a++) v[a] = __dadd_rn(v[a], __dmul_rn(fmm_f2d(f[a]), hk));
         }
-        int rt = target_rung(f[0], f[1], f[2], eps, dt0, R);
+        int rt = target_rung(f[0], f[1], f[2], eps, dt0, R, t0);
         int rn = rt;
         if (rt < r) {
             rn = rt;
@@ -131,18 +166,18 @@ __global__ void k_kick_drift_i32(unsigned int* __restrict__ ipos, float* __restr
         }
         r = rn;
         rung[i] = (unsigned char)r;
-        const double hk = ldexp(dt0, -r - 1);
+        const double hk = pow2_scale(dt0, r + 1);
         for (int a = 0; a < 3; a++) {
-            v[a] = __dadd_rn(v[a], __dmul_rn((double)f[a], hk));
-            v32[a] = __double2float_rn(v[a]);
+            v[a] = __dadd_rn(v[a], __dmul_rn(fmm_f2d(f[a]), hk));
+            v32[a] = fmm_d2f_rn(v[a]);
             vel[a * n + i] = v32[a];
         }
     }
-    const double h = ldexp(dt0, -R);
+    const double h = pow2_scale(dt0, R);
     long long u[3];
     bool out = false;
     for (int a = 0; a < 3; a++) {
-        const long long d = __double2ll_rn(__dmul_rn(__dmul_rn((double)v32[a], h), 4294967296.0));
+        const long long d = __double2ll_rn(__dmul_rn(__dmul_rn(fmm_f2d(v32[a]), h), 4294967296.0));
         u[a] = (long long)ipos[a * n + i] + d;
         if (periodic) u[a] &= 0xffffffffLL;
         else if (u[a] < 0 || u[a] > 0xffffffffLL) out = true;
@@ -161,14 +196,15 @@ cudaError_t fmm_launch_kick_drift_i32(unsigned int* ipos, float* vel, const floa
                                       int substep, int closing, int periodic, DevCounters* ctr, cudaStream_t s)
 {
     k_kick_drift_i32<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(ipos, vel, acc, rung, active_next, n, eps, dt0,
-                                                                    max_rung, substep, closing, periodic,
-                                                                    &ctr->kdk_status);
+                                                                    max_rung, rung_threshold(eps, dt0), substep, closing,
+                                                                    periodic, &ctr->kdk_status);
     return cudaGetLastError();
 }
 
 cudaError_t fmm_launch_assign_rungs(const float* acc, unsigned char* rung, long long n, double eps, double dt0,
                                     int max_rung, cudaStream_t s)
 {
-    k_assign_rungs<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(acc, rung, n, eps, dt0, max_rung);
+    k_assign_rungs<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(acc, rung, n, eps, dt0, max_rung,
+                                                                  rung_threshold(eps, dt0));
     return cudaGetLastError();
 }
