@@ -18,8 +18,11 @@
 
 cudaError_t fmm_mlp_pack(const float* params, unsigned char* packed, cudaStream_t s);
 cudaError_t fmm_mlp_grad(const float* params, const float* feats, const float* labels, const unsigned int* idx,
-                         long long nrows, float inv_b, float loss_scale, float* grad, float* loss, cudaStream_t s);
-cudaError_t fmm_mlp_adam(float* p, const float* g, float* m, float* v, float lr, int step, cudaStream_t s);
+                         long long nrows, float inv_b, float loss_scale, float* part, float* grad, float* loss,
+                         cudaStream_t s);
+cudaError_t fmm_mlp_adam(float* p, const float* feats, const float* labels, const unsigned int* idx, long long nrows,
+                         float inv_b, float loss_scale, float* part, float* m, float* v, float lr, int step, float* loss,
+                         cudaStream_t s);
 cudaError_t fmm_mlp_predict(const unsigned char* packed, const float* feats, long long n, float* out, cudaStream_t s);
 cudaError_t fmm_launch_audit_labels(DevTree& t, const int2* pairs, long long npairs, const float* acc_ref,
                                     long long n, float eps, float* feats, float* labels, cudaStream_t s);
@@ -143,7 +146,7 @@ struct fmm_ctx {
     long long cap_d = 0;
     int second_root = -1;
     // learned criterion: FP32 master parameters, Adam state, packed BF16 copy
-    float *mlp_p = nullptr, *mlp_g = nullptr, *mlp_m = nullptr, *mlp_v = nullptr, *mlp_loss = nullptr;
+    float *mlp_p = nullptr, *mlp_g = nullptr, *mlp_m = nullptr, *mlp_v = nullptr, *mlp_loss = nullptr, *mlp_part = nullptr;
     unsigned char* mlp_packed = nullptr;
     bool mlp_ready = false;
     int2* audit_pairs = nullptr;
@@ -289,7 +292,7 @@ static void free_all(fmm_ctx* c)
     if (t.box_off_h) cudaFreeHost(t.box_off_h);
     if (c->totals_h) cudaFreeHost(c->totals_h);
     void* hs[] = {c->hpos, c->hmass, c->hacc, c->hpot, c->hact, c->mlp_p, c->mlp_g, c->mlp_m, c->mlp_v, c->mlp_loss,
-                  c->mlp_packed, c->audit_pairs, c->mlp_idx, c->mlp_pred};
+                  c->mlp_part, c->mlp_packed, c->audit_pairs, c->mlp_idx, c->mlp_pred};
     for (void* p : hs) dev_free(p);
     for (auto& e : c->ev)
         if (e) cudaEventDestroy(e);
@@ -317,7 +320,7 @@ extern "C" fmm_status fmm_memory_info(const fmm_ctx* c, long long* device_bytes,
     long long d = 0;
     for (void* p : tree_walk_buffers(c)) d += (long long)dev_size(p);
     const void* hs[] = {c->hpos, c->hmass, c->hacc, c->hpot, c->hact, c->mlp_p, c->mlp_g, c->mlp_m, c->mlp_v,
-                        c->mlp_loss, c->mlp_packed, c->audit_pairs, c->mlp_idx, c->mlp_pred};
+                        c->mlp_loss, c->mlp_part, c->mlp_packed, c->audit_pairs, c->mlp_idx, c->mlp_pred};
     for (const void* p : hs) d += (long long)dev_size(p);
     d += (long long)(sizeof(DevCounters) + 12 * sizeof(unsigned int));
     if (device_bytes) *device_bytes = d;
@@ -1991,6 +1994,13 @@ static fmm_status mlp_alloc(fmm_ctx* c)
     return FMM_OK;
 }
 
+// the training kernels' partial sums
+static fmm_status mlp_part_alloc(fmm_ctx* c)
+{
+    if (!c->mlp_part) CK(alloc(&c->mlp_part, (long long)MLP_GRAD_BLOCKS * MLP_PART));
+    return FMM_OK;
+}
+
 extern "C" fmm_status fmm_mlp_load(fmm_ctx* c, const float* params, long long n)
 {
     if (!c || !params) return fail(FMM_ERR_ARG, "NULL argument");
@@ -2037,10 +2047,11 @@ extern "C" fmm_status fmm_mlp_gradient(fmm_ctx* c, const float* feats, const flo
     if (n < 1) return fail(FMM_ERR_ARG, "n must be >= 1");
     if (!c->mlp_ready) return fail(FMM_ERR_STATE, "no network parameters");
     CK(cudaSetDevice(c->device));
-    CK(cudaMemsetAsync(c->mlp_g, 0, sizeof(float) * MLP_NW, c->stream));
+    fmm_status st = mlp_part_alloc(c);
+    if (st != FMM_OK) return st;
     CK(cudaMemsetAsync(c->mlp_loss, 0, sizeof(float), c->stream));
-    CK(fmm_mlp_grad(c->mlp_p, feats, labels, nullptr, n, 1.0f / (float)n, 1.0f / (float)n, c->mlp_g, c->mlp_loss,
-                    c->stream));
+    CK(fmm_mlp_grad(c->mlp_p, feats, labels, nullptr, n, 1.0f / (float)n, 1.0f / (float)n, c->mlp_part, c->mlp_g,
+                    c->mlp_loss, c->stream));
     CK(cudaMemcpyAsync(grad, c->mlp_g, sizeof(float) * MLP_NW, cudaMemcpyDeviceToHost, c->stream));
     if (loss) CK(cudaMemcpyAsync(loss, c->mlp_loss, sizeof(float), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -2068,6 +2079,7 @@ extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float*
     CK(cudaSetDevice(c->device));
     cudaStream_t s = c->stream;
     fmm_status st = mlp_alloc(c);
+    if (st == FMM_OK) st = mlp_part_alloc(c);
     if (st != FMM_OK) return st;
     // normalisation from the data, weights from the seed
     std::vector<float> hf((size_t)n * MLP_F), hl((size_t)n);
@@ -2119,11 +2131,9 @@ extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float*
         CK(cudaMemsetAsync(c->mlp_loss, 0, sizeof(float), s));
         for (long long b = 0; b < n; b += batch) {
             const long long nr = std::min<long long>(batch, n - b);
-            CK(cudaMemsetAsync(c->mlp_g, 0, sizeof(float) * MLP_NW, s));
             // minibatch-mean gradient; the loss is accumulated as the epoch mean
-            CK(fmm_mlp_grad(c->mlp_p, feats, labels, c->mlp_idx + b, nr, 1.0f / (float)nr, 1.0f / (float)n, c->mlp_g,
-                            c->mlp_loss, s));
-            CK(fmm_mlp_adam(c->mlp_p, c->mlp_g, c->mlp_m, c->mlp_v, lr, ++step, s));
+            CK(fmm_mlp_adam(c->mlp_p, feats, labels, c->mlp_idx + b, nr, 1.0f / (float)nr, 1.0f / (float)n, c->mlp_part,
+                            c->mlp_m, c->mlp_v, lr, ++step, c->mlp_loss, s));
         }
         CK(cudaMemcpyAsync(&last, c->mlp_loss, sizeof(float), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));

@@ -3,6 +3,8 @@
 // criterion is the fixed-theta test of Sec. 3.1; see mlp.cuh for the network.
 #include <math.h>
 
+#include <algorithm>
+
 #include "expansions.cuh"
 #include "fmm_internal.cuh"
 #include "mlp.cuh"
@@ -50,156 +52,274 @@ cudaError_t fmm_mlp_pack(const float* params, unsigned char* packed, cudaStream_
 
 // ---------------------------------------------------------------- training (FP32)
 
-// Gradient of 0.5 * mean((y - label)^2) over a minibatch, accumulated into grad with atomics.
-// One block of 64 threads per 64 rows: thread j owns hidden unit j in the forward pass and
-// row j of each weight gradient in the backward pass; activations live in shared memory.
-#define TB_ROWS 64
-#define TPAD 65
-__global__ void __launch_bounds__(64) k_mlp_grad(const float* __restrict__ p, const float* __restrict__ feats,
-                                                 const float* __restrict__ labels, const unsigned int* __restrict__ idx,
-                                                 long long nrows, float inv_b, float loss_scale,
-                                                 float* __restrict__ grad, float* __restrict__ loss)
+// Gradient of 0.5 * mean((y - label)^2) over a minibatch.  A block takes tiles of 64 rows and keeps its
+// weight gradients in registers over them; its sums go to a slot of its own, and k_mlp_step adds the
+// slots in order, so the weights of a training run are a function of its inputs.  (The loss is summed row by row
+// with atomics.)
+//
+// The six products of a tile (two hidden layers forward, their deltas, their weight gradients) are
+// 64 wide and run from shared memory: 2 rows x 4 units per thread forward and for the deltas, 2 x 4
+// weights per thread for the gradients, operands as float4 (6 loads for 32 multiply-adds, 2 for 8).
+// Both hidden matrices lie there twice, as stored and transposed, so that either product reads along
+// its output.  FP32 throughout, every sum in the order of its index.  Bound by its shared-memory loads
+// and the chain of layers: a minibatch of 4096 rows is 64 blocks of one tile.  One thread per hidden
+// unit, two warps a block, with the weights read from global memory and the gradients added with
+// atomics took 252 us for it.
+#define GR_ROWS 64
+#define GR_THREADS 512
+#define GR_PAD 68  // row stride of the activations and weights in shared memory
+struct GradSmem {
+    float W2t[MLP_H * GR_PAD], W3t[MLP_H * GR_PAD];  // [k][j], forward
+    float W2[MLP_H * GR_PAD], W3[MLP_H * GR_PAD];    // [i][j], deltas
+    float W1t[MLP_F * GR_PAD];
+    float H1[GR_ROWS * GR_PAD], H2[GR_ROWS * GR_PAD], H3[GR_ROWS * GR_PAD];
+    float Da[GR_ROWS * GR_PAD], Db[GR_ROWS * GR_PAD];
+    float X[GR_ROWS * MLP_F];
+    float b1[MLP_H], b2[MLP_H], b3[MLP_H], zero[MLP_H], w4[MLP_H];
+    float dy[GR_ROWS];
+};
+
+// out[s][j] = f(b[j] + sum_k in[s][k] Wt[k][j]), f the ReLU, or (MASK) zero where mask[s][j] is not > 0
+template <int K, int KSTRIDE, bool MASK>
+__device__ __forceinline__ void grad_layer(const float* __restrict__ in, const float* __restrict__ Wt,
+                                           const float* __restrict__ b, const float* __restrict__ mask,
+                                           float* __restrict__ out, int tid)
 {
-    extern __shared__ float sm[];
-    float* X = sm;                         // [64][8]
-    float* H1 = X + TB_ROWS * MLP_F;       // [64][65]
-    float* H2 = H1 + TB_ROWS * TPAD;
-    float* H3 = H2 + TB_ROWS * TPAD;
-    float* Da = H3 + TB_ROWS * TPAD;
-    float* Db = Da + TB_ROWS * TPAD;
-    float* dy = Db + TB_ROWS * TPAD;       // [64]
-    const int j = threadIdx.x;
-    const long long r0 = (long long)blockIdx.x * TB_ROWS;
-    const int nr = (int)min((long long)TB_ROWS, nrows - r0);
-    // inputs
-    if (j < nr) {
-        const unsigned int r = idx ? idx[r0 + j] : (unsigned int)(r0 + j);
-        for (int k = 0; k < MLP_F; k++) X[j * MLP_F + k] = (feats[(long long)r * MLP_F + k] - p[MLP_MEAN + k]) * p[MLP_ISTD + k];
-        dy[j] = labels[r];
-    } else {
-        for (int k = 0; k < MLP_F; k++) X[j * MLP_F + k] = 0.0f;
-        dy[j] = 0.0f;
-    }
-    __syncthreads();
-    // forward: unit j of each layer for all rows
-    {
-        float w[MLP_F];
-        for (int k = 0; k < MLP_F; k++) w[k] = p[MLP_W1 + j * MLP_F + k];
-        const float b = p[MLP_B1 + j];
-        for (int s = 0; s < TB_ROWS; s++) {
-            float z = b;
-            for (int k = 0; k < MLP_F; k++) z = fmaf(w[k], X[s * MLP_F + k], z);
-            H1[s * TPAD + j] = fmaxf(z, 0.0f);
+    const int r0 = (tid >> 4) * 2, j0 = (tid & 15) * 4;
+    const float4 bv = *reinterpret_cast<const float4*>(b + j0);
+    float4 z0 = bv, z1 = bv;
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+        const float4 h0 = *reinterpret_cast<const float4*>(in + r0 * KSTRIDE + k);
+        const float4 h1 = *reinterpret_cast<const float4*>(in + (r0 + 1) * KSTRIDE + k);
+        const float a0[4] = {h0.x, h0.y, h0.z, h0.w}, a1[4] = {h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const float4 w = *reinterpret_cast<const float4*>(Wt + (k + q) * GR_PAD + j0);
+            z0.x = fmaf(w.x, a0[q], z0.x);
+            z0.y = fmaf(w.y, a0[q], z0.y);
+            z0.z = fmaf(w.z, a0[q], z0.z);
+            z0.w = fmaf(w.w, a0[q], z0.w);
+            z1.x = fmaf(w.x, a1[q], z1.x);
+            z1.y = fmaf(w.y, a1[q], z1.y);
+            z1.z = fmaf(w.z, a1[q], z1.z);
+            z1.w = fmaf(w.w, a1[q], z1.w);
         }
     }
-    __syncthreads();
-    const float* Ws[2] = {p + MLP_W2, p + MLP_W3};
-    const float* Bs[2] = {p + MLP_B2, p + MLP_B3};
-    float* Hin[2] = {H1, H2};
-    float* Hout[2] = {H2, H3};
-    for (int l = 0; l < 2; l++) {
-        const float* W = Ws[l] + j * MLP_H;
-        const float b = Bs[l][j];
-        for (int s = 0; s < TB_ROWS; s++) {
-            float z = b;
-            for (int k = 0; k < MLP_H; k++) z = fmaf(__ldg(W + k), Hin[l][s * TPAD + k], z);
-            Hout[l][s * TPAD + j] = fmaxf(z, 0.0f);
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        float4 z = h ? z1 : z0;
+        float* const o = out + (r0 + h) * GR_PAD + j0;
+        if (MASK) {
+            const float4 m = *reinterpret_cast<const float4*>(mask + (r0 + h) * GR_PAD + j0);
+            z = make_float4(m.x > 0.0f ? z.x : 0.0f, m.y > 0.0f ? z.y : 0.0f, m.z > 0.0f ? z.z : 0.0f,
+                            m.w > 0.0f ? z.w : 0.0f);
+        } else {
+            z = make_float4(fmaxf(z.x, 0.0f), fmaxf(z.y, 0.0f), fmaxf(z.z, 0.0f), fmaxf(z.w, 0.0f));
         }
-        __syncthreads();
+        *reinterpret_cast<float4*>(o) = z;
     }
-    // output and its error (thread j = row j)
-    {
-        float y = p[MLP_B4];
-        for (int k = 0; k < MLP_H; k++) y = fmaf(p[MLP_W4 + k], H3[j * TPAD + k], y);
-        const float r = j < nr ? y - dy[j] : 0.0f;
-        if (j < nr) atomicAdd(loss, 0.5f * r * r * loss_scale);
-        __syncthreads();
-        dy[j] = r * inv_b;
-    }
-    __syncthreads();
-    // output layer gradient; delta of layer 3 into Da
-    {
-        float gw = 0.0f, gb = 0.0f;
-        const float w4 = p[MLP_W4 + j];
-        for (int s = 0; s < TB_ROWS; s++) {
-            gw = fmaf(H3[s * TPAD + j], dy[s], gw);
-            Da[s * TPAD + j] = H3[s * TPAD + j] > 0.0f ? dy[s] * w4 : 0.0f;
-            gb += dy[s];
-        }
-        atomicAdd(grad + MLP_W4 + j, gw);
-        if (j == 0) atomicAdd(grad + MLP_B4, gb);
-    }
-    __syncthreads();
-    // hidden layers 3 and 2: dW[j][k] = sum_s D[s][j] Hin[s][k]; delta_in[s][j] = sum_i D[s][i] W[i][j] (Hin > 0)
-    const int offW[2] = {MLP_W3, MLP_W2}, offB[2] = {MLP_B3, MLP_B2};
-    float* Hprev[2] = {H2, H1};
-    float* Din[2] = {Da, Db};
-    float* Dout[2] = {Db, Da};
-    for (int l = 0; l < 2; l++) {
-        const float* D = Din[l];
-        const float* Hp = Hprev[l];
-        float gb = 0.0f;
-        for (int s = 0; s < TB_ROWS; s++) gb += D[s * TPAD + j];
-        atomicAdd(grad + offB[l] + j, gb);
-        for (int k = 0; k < MLP_H; k++) {
-            float gw = 0.0f;
-            for (int s = 0; s < TB_ROWS; s++) gw = fmaf(D[s * TPAD + j], Hp[s * TPAD + k], gw);
-            atomicAdd(grad + offW[l] + j * MLP_H + k, gw);
-        }
-        const float* W = p + offW[l];
-        for (int s = 0; s < TB_ROWS; s++) {
-            float a = 0.0f;
-            for (int i = 0; i < MLP_H; i++) a = fmaf(D[s * TPAD + i], __ldg(W + i * MLP_H + j), a);
-            Dout[l][s * TPAD + j] = Hp[s * TPAD + j] > 0.0f ? a : 0.0f;
-        }
-        __syncthreads();
-    }
-    // first layer: delta in Da (after two swaps)
-    {
-        const float* D = Da;
-        float gb = 0.0f;
-        for (int s = 0; s < TB_ROWS; s++) gb += D[s * TPAD + j];
-        atomicAdd(grad + MLP_B1 + j, gb);
-        for (int k = 0; k < MLP_F; k++) {
-            float gw = 0.0f;
-            for (int s = 0; s < TB_ROWS; s++) gw = fmaf(D[s * TPAD + j], X[s * MLP_F + k], gw);
-            atomicAdd(grad + MLP_W1 + j * MLP_F + k, gw);
+}
+
+// g[a][c] += sum_s D[s][j0 + a] H[s][k0 + c]
+__device__ __forceinline__ void grad_weights(const float* __restrict__ D, const float* __restrict__ H, float g[2][4],
+                                             int tid)
+{
+    const int j0 = (tid >> 4) * 2, k0 = (tid & 15) * 4;
+#pragma unroll 4
+    for (int s = 0; s < GR_ROWS; s++) {
+        const float2 d = *reinterpret_cast<const float2*>(D + s * GR_PAD + j0);
+        const float4 h = *reinterpret_cast<const float4*>(H + s * GR_PAD + k0);
+        const float dv[2] = {d.x, d.y};
+#pragma unroll
+        for (int a = 0; a < 2; a++) {
+            g[a][0] = fmaf(dv[a], h.x, g[a][0]);
+            g[a][1] = fmaf(dv[a], h.y, g[a][1]);
+            g[a][2] = fmaf(dv[a], h.z, g[a][2]);
+            g[a][3] = fmaf(dv[a], h.w, g[a][3]);
         }
     }
 }
 
-static size_t grad_smem() { return (size_t)(TB_ROWS * MLP_F + 5 * TB_ROWS * TPAD + TB_ROWS) * sizeof(float); }
-
-cudaError_t fmm_mlp_grad(const float* params, const float* feats, const float* labels, const unsigned int* idx,
-                         long long nrows, float inv_b, float loss_scale, float* grad, float* loss, cudaStream_t s)
+__global__ void __launch_bounds__(GR_THREADS) k_mlp_grad(const float* __restrict__ p, const float* __restrict__ feats,
+                                                         const float* __restrict__ labels,
+                                                         const unsigned int* __restrict__ idx, long long nrows,
+                                                         float inv_b, float loss_scale, float* __restrict__ part,
+                                                         float* __restrict__ loss)
 {
-    static std::atomic<unsigned long long> attr{0};
-    cudaError_t e = fmm_smem_attr_once(k_mlp_grad, (int)grad_smem(), attr);
-    if (e != cudaSuccess) return e;
-    k_mlp_grad<<<(unsigned)fmm_ceil_div(nrows, TB_ROWS), 64, grad_smem(), s>>>(params, feats, labels, idx, nrows, inv_b,
-                                                                             loss_scale, grad, loss);
-    return cudaGetLastError();
+    extern __shared__ __align__(16) unsigned char gsm[];
+    GradSmem& S = *reinterpret_cast<GradSmem*>(gsm);
+    const int tid = threadIdx.x;
+    for (int i = tid; i < MLP_H * MLP_H; i += GR_THREADS) {
+        const int j = i >> 6, k = i & 63;
+        const float w2 = p[MLP_W2 + i], w3 = p[MLP_W3 + i];
+        S.W2[j * GR_PAD + k] = w2;
+        S.W2t[k * GR_PAD + j] = w2;
+        S.W3[j * GR_PAD + k] = w3;
+        S.W3t[k * GR_PAD + j] = w3;
+    }
+    for (int i = tid; i < MLP_H * MLP_F; i += GR_THREADS) S.W1t[(i & 7) * GR_PAD + (i >> 3)] = p[MLP_W1 + i];
+    if (tid < MLP_H) {
+        S.b1[tid] = p[MLP_B1 + tid];
+        S.b2[tid] = p[MLP_B2 + tid];
+        S.b3[tid] = p[MLP_B3 + tid];
+        S.w4[tid] = p[MLP_W4 + tid];
+        S.zero[tid] = 0.0f;
+    }
+    // this thread's gradients: 2 x 4 of each hidden matrix, one of the first, one of the four vectors
+    float g2[2][4] = {}, g3[2][4] = {}, g1 = 0.0f, gv = 0.0f, gb4 = 0.0f;
+    const int vj = tid & 63, vq = tid >> 6;  // vector gradient: b1, b2, b3, w4 of unit vj
+    const long long tiles = fmm_ceil_div(nrows, GR_ROWS);
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const long long r0 = tile * GR_ROWS;
+        const int nr = (int)min((long long)GR_ROWS, nrows - r0);
+        __syncthreads();
+        {
+            const int s = tid >> 3, k = tid & 7;  // one feature per thread
+            float x = 0.0f;
+            if (s < nr) {
+                const unsigned int r = idx ? idx[r0 + s] : (unsigned int)(r0 + s);
+                x = (feats[(long long)r * MLP_F + k] - p[MLP_MEAN + k]) * p[MLP_ISTD + k];
+                if (k == 0) S.dy[s] = labels[r];
+            }
+            S.X[s * MLP_F + k] = x;
+        }
+        __syncthreads();
+        grad_layer<MLP_F, MLP_F, false>(S.X, S.W1t, S.b1, nullptr, S.H1, tid);
+        __syncthreads();
+        grad_layer<MLP_H, GR_PAD, false>(S.H1, S.W2t, S.b2, nullptr, S.H2, tid);
+        __syncthreads();
+        grad_layer<MLP_H, GR_PAD, false>(S.H2, S.W3t, S.b3, nullptr, S.H3, tid);
+        __syncthreads();
+        if (tid < GR_ROWS) {
+            // output and its error, a row per lane, summed in the order of the units
+            float y = p[MLP_B4];
+#pragma unroll 8
+            for (int k = 0; k < MLP_H; k += 4) {
+                const float4 w = *reinterpret_cast<const float4*>(S.w4 + k);
+                const float4 h = *reinterpret_cast<const float4*>(S.H3 + tid * GR_PAD + k);
+                y = fmaf(w.w, h.w, fmaf(w.z, h.z, fmaf(w.y, h.y, fmaf(w.x, h.x, y))));
+            }
+            const float r = tid < nr ? y - S.dy[tid] : 0.0f;
+            if (tid < nr) atomicAdd(loss, 0.5f * r * r * loss_scale);
+            S.dy[tid] = r * inv_b;
+        }
+        __syncthreads();
+        // delta of layer 3
+        for (int i = tid; i < GR_ROWS * MLP_H; i += GR_THREADS) {
+            const int s = i >> 6, j = i & 63;
+            S.Da[s * GR_PAD + j] = S.H3[s * GR_PAD + j] > 0.0f ? S.dy[s] * S.w4[j] : 0.0f;
+        }
+        __syncthreads();
+        if (vq == 3) {
+            for (int s = 0; s < GR_ROWS; s++) gv = fmaf(S.H3[s * GR_PAD + vj], S.dy[s], gv);
+            if (vj == 0)
+                for (int s = 0; s < GR_ROWS; s++) gb4 += S.dy[s];
+        } else if (vq == 2) {
+            for (int s = 0; s < GR_ROWS; s++) gv += S.Da[s * GR_PAD + vj];
+        }
+        grad_weights(S.Da, S.H2, g3, tid);
+        grad_layer<MLP_H, GR_PAD, true>(S.Da, S.W3, S.zero, S.H2, S.Db, tid);
+        __syncthreads();
+        if (vq == 1)
+            for (int s = 0; s < GR_ROWS; s++) gv += S.Db[s * GR_PAD + vj];
+        grad_weights(S.Db, S.H1, g2, tid);
+        grad_layer<MLP_H, GR_PAD, true>(S.Db, S.W2, S.zero, S.H1, S.Da, tid);
+        __syncthreads();
+        if (vq == 0)
+            for (int s = 0; s < GR_ROWS; s++) gv += S.Da[s * GR_PAD + vj];
+        {
+            const int j = tid >> 3, k = tid & 7;
+            for (int s = 0; s < GR_ROWS; s++) g1 = fmaf(S.Da[s * GR_PAD + j], S.X[s * MLP_F + k], g1);
+        }
+    }
+    // the block's sums in its slot, in the order of the parameters, then its loss
+    float* const out = part + (long long)blockIdx.x * MLP_PART;
+    {
+        const int j0 = (tid >> 4) * 2, k0 = (tid & 15) * 4;
+#pragma unroll
+        for (int a = 0; a < 2; a++)
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                out[MLP_W2 + (j0 + a) * MLP_H + k0 + c] = g2[a][c];
+                out[MLP_W3 + (j0 + a) * MLP_H + k0 + c] = g3[a][c];
+            }
+        out[MLP_W1 + tid] = g1;
+        if (vq < 4) out[(vq == 0 ? MLP_B1 : vq == 1 ? MLP_B2 : vq == 2 ? MLP_B3 : MLP_W4) + vj] = gv;
+        if (tid == 3 * 64) out[MLP_B4] = gb4;
+    }
 }
 
-// Adam step on the trainable weights (bias-corrected moments)
-__global__ void k_mlp_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                           float* __restrict__ v, float lr, float b1, float b2, float eps, float c1, float c2)
+// Adds the blocks' sums in order: the gradient, written to grad, or taken at once by an Adam step on the
+// trainable weights (bias-corrected moments).
+struct AdamArgs {
+    float *p, *m, *v;
+    float lr, b1, b2, eps, c1, c2;
+};
+template <bool ADAM>
+__global__ void __launch_bounds__(64) k_mlp_step(const float* __restrict__ part, int nb, float* __restrict__ grad,
+                                                 AdamArgs a)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MLP_NW) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    float gi = 0.0f;
+#pragma unroll 16
+    for (int b = 0; b < nb; b++) gi += part[(long long)b * MLP_PART + i];
+    if (!ADAM) {
+        grad[i] = gi;
+        return;
+    }
+    const float mi = a.b1 * a.m[i] + (1.0f - a.b1) * gi;
+    const float vi = a.b2 * a.v[i] + (1.0f - a.b2) * gi * gi;
+    a.m[i] = mi;
+    a.v[i] = vi;
+    a.p[i] -= a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + a.eps);
 }
 
-cudaError_t fmm_mlp_adam(float* p, const float* g, float* m, float* v, float lr, int step, cudaStream_t s)
+static cudaError_t launch_grad(const float* params, const float* feats, const float* labels, const unsigned int* idx,
+                               long long nrows, float inv_b, float loss_scale, float* part, float* loss, int* nb,
+                               cudaStream_t s)
 {
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);
-    k_mlp_adam<<<(MLP_NW + 255) / 256, 256, 0, s>>>(p, g, m, v, lr, b1, b2, 1e-8f, c1, c2);
+    static std::atomic<unsigned long long> attr{0};
+    cudaError_t e = fmm_smem_attr_once(k_mlp_grad, (int)sizeof(GradSmem), attr);
+    if (e != cudaSuccess) return e;
+    *nb = (int)std::min<long long>(fmm_ceil_div(nrows, GR_ROWS), MLP_GRAD_BLOCKS);
+    k_mlp_grad<<<*nb, GR_THREADS, sizeof(GradSmem), s>>>(params, feats, labels, idx, nrows, inv_b, loss_scale, part,
+                                                              loss);
+    return cudaGetLastError();
+}
+
+// grad (MLP_NW values) of the rows, and their loss added to *loss; part: MLP_GRAD_BLOCKS * MLP_PART floats
+cudaError_t fmm_mlp_grad(const float* params, const float* feats, const float* labels, const unsigned int* idx,
+                         long long nrows, float inv_b, float loss_scale, float* part, float* grad, float* loss,
+                         cudaStream_t s)
+{
+    int nb = 0;
+    cudaError_t e = launch_grad(params, feats, labels, idx, nrows, inv_b, loss_scale, part, loss, &nb, s);
+    if (e != cudaSuccess) return e;
+    k_mlp_step<false><<<(MLP_NW + 63) / 64, 64, 0, s>>>(part, nb, grad, AdamArgs{});
+    return cudaGetLastError();
+}
+
+// one Adam step on the rows' gradient; their loss is added to *loss
+cudaError_t fmm_mlp_adam(float* p, const float* feats, const float* labels, const unsigned int* idx, long long nrows,
+                         float inv_b, float loss_scale, float* part, float* m, float* v, float lr, int step, float* loss,
+                         cudaStream_t s)
+{
+    int nb = 0;
+    cudaError_t e = launch_grad(p, feats, labels, idx, nrows, inv_b, loss_scale, part, loss, &nb, s);
+    if (e != cudaSuccess) return e;
+    AdamArgs a;
+    a.p = p;
+    a.m = m;
+    a.v = v;
+    a.lr = lr;
+    a.b1 = 0.9f;
+    a.b2 = 0.999f;
+    a.eps = 1e-8f;
+    a.c1 = 1.0f - powf(a.b1, (float)step);
+    a.c2 = 1.0f - powf(a.b2, (float)step);
+    k_mlp_step<true><<<(MLP_NW + 63) / 64, 64, 0, s>>>(part, nb, nullptr, a);
     return cudaGetLastError();
 }
 

@@ -33,6 +33,11 @@
 #define MLP_SUR (MLP_ISTD + MLP_F)
 #define MLP_NP (MLP_SUR + MLP_NSUR)  // 8989 parameters in all
 
+// training: a block's slot of partial sums (the weights' gradients, padding), and the most
+// blocks a gradient takes (one per SM)
+#define MLP_PART (MLP_NW + 3)
+#define MLP_GRAD_BLOCKS 152
+
 // packed inference layout (bytes), identical in global and shared memory; matrix rows are
 // padded (24 / 72 BF16) so the fragment loads of the 8 row groups hit distinct banks
 #define MLPP_W1 0        // [64][24] bf16, columns 8..23 zero
