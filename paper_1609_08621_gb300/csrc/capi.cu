@@ -7,6 +7,7 @@
 #include <cmath>
 #include <string>
 #include <mutex>
+#include <thread>
 #include <unordered_map>
 #include <vector>
 
@@ -2068,6 +2069,31 @@ unsigned long long splitmix(unsigned long long& s)
     return z ^ (z >> 31);
 }
 double uniform01(unsigned long long& s) { return (double)(splitmix(s) >> 11) * (1.0 / 9007199254740992.0); }
+
+// Training's passes over its rows on the host (means, variances, the surrogate's normal equations and
+// residuals) were 20 of the 27 ms that 200k rows and 2 epochs took; in parts on several threads, with
+// the shuffles beside the GPU's epochs, the whole takes 11 ms.
+// f(chunk, begin, end) over HOST_CHUNKS equal parts of [0, n), on several threads where there are rows
+// enough to pay for starting them (about 10 us each against 20 ns a row).  The parts are the same
+// whatever runs them, so sums formed per part and added in their order do not depend on the machine.
+constexpr int HOST_CHUNKS = 16;
+template <class F>
+void host_chunks(long long n, F f)
+{
+    auto part = [&](int k) { f(k, n * k / HOST_CHUNKS, n * (k + 1) / HOST_CHUNKS); };
+    std::vector<std::thread> threads;
+    int k = 1;
+    if (n >= 16384) {
+        try {
+            threads.reserve(HOST_CHUNKS);
+            for (; k < HOST_CHUNKS; k++) threads.emplace_back(part, k);
+        } catch (...) {  // no thread to be had: the rest runs here
+        }
+    }
+    part(0);
+    for (; k < HOST_CHUNKS; k++) part(k);
+    for (std::thread& t : threads) t.join();
+}
 }  // namespace
 
 extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float* labels, long long n, int epochs,
@@ -2087,17 +2113,35 @@ extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float*
     CK(cudaMemcpyAsync(hl.data(), labels, sizeof(float) * hl.size(), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     std::vector<float> p(MLP_NP, 0.0f);
-    double lmean = 0.0;
-    for (long long i = 0; i < n; i++) lmean += hl[i];
-    lmean /= (double)n;
+    double mean[MLP_F + 1] = {}, var[MLP_F] = {};  // of the features, and the labels' mean last
+    {
+        double sum[HOST_CHUNKS][MLP_F + 1] = {};
+        host_chunks(n, [&](int q, long long b, long long e) {
+            double t[MLP_F + 1] = {};
+            for (long long i = b; i < e; i++) {
+                for (int k = 0; k < MLP_F; k++) t[k] += hf[i * MLP_F + k];
+                t[MLP_F] += hl[i];
+            }
+            std::copy(t, t + MLP_F + 1, sum[q]);
+        });
+        for (int k = 0; k <= MLP_F; k++) {
+            for (int q = 0; q < HOST_CHUNKS; q++) mean[k] += sum[q][k];
+            mean[k] /= (double)n;
+        }
+        host_chunks(n, [&](int q, long long b, long long e) {
+            double t[MLP_F] = {};
+            for (long long i = b; i < e; i++)
+                for (int k = 0; k < MLP_F; k++) t[k] += (hf[i * MLP_F + k] - mean[k]) * (hf[i * MLP_F + k] - mean[k]);
+            std::copy(t, t + MLP_F, sum[q]);
+        });
+        for (int k = 0; k < MLP_F; k++) {
+            for (int q = 0; q < HOST_CHUNKS; q++) var[k] += sum[q][k];
+            var[k] /= (double)n;
+        }
+    }
     for (int k = 0; k < MLP_F; k++) {
-        double m = 0.0, v = 0.0;
-        for (long long i = 0; i < n; i++) m += hf[i * MLP_F + k];
-        m /= (double)n;
-        for (long long i = 0; i < n; i++) v += (hf[i * MLP_F + k] - m) * (hf[i * MLP_F + k] - m);
-        v /= (double)n;
-        p[MLP_MEAN + k] = (float)m;
-        p[MLP_ISTD + k] = (float)(v > 1e-20 ? 1.0 / sqrt(v) : 1.0);
+        p[MLP_MEAN + k] = (float)mean[k];
+        p[MLP_ISTD + k] = (float)(var[k] > 1e-20 ? 1.0 / sqrt(var[k]) : 1.0);
     }
     unsigned long long rs = 0x5eedull ^ ((unsigned long long)seed << 17);
     auto init = [&](int off, int rows, int cols) {
@@ -2109,7 +2153,7 @@ extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float*
     init(MLP_W3, MLP_H, MLP_H);
     init(MLP_W4, 1, MLP_H);
     for (int i = 0; i < MLP_H; i++) p[MLP_W4 + i] *= 0.1f;
-    p[MLP_B4] = (float)lmean;
+    p[MLP_B4] = (float)mean[MLP_F];
     CK(cudaMemcpyAsync(c->mlp_p, p.data(), sizeof(float) * MLP_NP, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(c->mlp_m, 0, sizeof(float) * MLP_NW, s));
     CK(cudaMemsetAsync(c->mlp_v, 0, sizeof(float) * MLP_NW, s));
@@ -2118,22 +2162,33 @@ extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float*
         CK(alloc(&c->mlp_idx, n));
         c->mlp_idx_cap = n;
     }
-    std::vector<unsigned int> perm((size_t)n);
-    for (long long i = 0; i < n; i++) perm[i] = (unsigned int)i;
+    // an epoch's order is shuffled from the last one's while the GPU runs that one, into the other of two
+    // buffers (the copy to the device may still read the first)
+    std::vector<unsigned int> perm[2];
+    perm[0].resize((size_t)n);
+    for (long long i = 0; i < n; i++) perm[0][i] = (unsigned int)i;
+    auto shuffle = [&](std::vector<unsigned int>& v) {
+        for (long long i = n - 1; i > 0; i--) {  // Fisher-Yates
+            long long j = (long long)(splitmix(rs) % (unsigned long long)(i + 1));
+            std::swap(v[i], v[j]);
+        }
+    };
+    shuffle(perm[0]);
     int step = 0;
     float last = 0.0f;
     for (int ep = 0; ep < epochs; ep++) {
-        for (long long i = n - 1; i > 0; i--) {  // Fisher-Yates
-            long long j = (long long)(splitmix(rs) % (unsigned long long)(i + 1));
-            std::swap(perm[i], perm[j]);
-        }
-        CK(cudaMemcpyAsync(c->mlp_idx, perm.data(), sizeof(unsigned int) * (size_t)n, cudaMemcpyHostToDevice, s));
+        const std::vector<unsigned int>& order = perm[ep & 1];
+        CK(cudaMemcpyAsync(c->mlp_idx, order.data(), sizeof(unsigned int) * (size_t)n, cudaMemcpyHostToDevice, s));
         CK(cudaMemsetAsync(c->mlp_loss, 0, sizeof(float), s));
         for (long long b = 0; b < n; b += batch) {
             const long long nr = std::min<long long>(batch, n - b);
             // minibatch-mean gradient; the loss is accumulated as the epoch mean
             CK(fmm_mlp_adam(c->mlp_p, feats, labels, c->mlp_idx + b, nr, 1.0f / (float)nr, 1.0f / (float)n, c->mlp_part,
                             c->mlp_m, c->mlp_v, lr, ++step, c->mlp_loss, s));
+        }
+        if (ep + 1 < epochs) {
+            perm[(ep + 1) & 1] = order;
+            shuffle(perm[(ep + 1) & 1]);
         }
         CK(cudaMemcpyAsync(&last, c->mlp_loss, sizeof(float), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -2163,29 +2218,47 @@ extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float*
             if (!isfinite(x[k])) return false;
         return isfinite((double)hl[i]) && isfinite((double)pred[i]);
     };
+    // sums over the rows, per part of them and then in the parts' order
     std::vector<double> scale(NC, 0.0);
     double cnt = 0;
     {
-        double x[2 + MLP_F];
-        for (long long i = 0; i < n; i++) {
-            if (!columns(i, x)) continue;
-            for (int k = 0; k < NC; k++) scale[k] += x[k] * x[k];
-            cnt += 1;
+        std::vector<double> sum((size_t)HOST_CHUNKS * (NC + 1), 0.0);
+        host_chunks(n, [&](int q, long long b, long long e) {
+            double x[2 + MLP_F], t[3 + MLP_F] = {};
+            for (long long i = b; i < e; i++) {
+                if (!columns(i, x)) continue;
+                for (int k = 0; k < NC; k++) t[k] += x[k] * x[k];
+                t[NC] += 1;
+            }
+            std::copy(t, t + NC + 1, sum.begin() + (size_t)q * (NC + 1));
+        });
+        for (int q = 0; q < HOST_CHUNKS; q++) {
+            for (int k = 0; k < NC; k++) scale[k] += sum[(size_t)q * (NC + 1) + k];
+            cnt += sum[(size_t)q * (NC + 1) + NC];
         }
     }
     float sur[MLP_NSUR] = {};  // off unless the fit is well posed
     if (cnt > 100) {
         for (int k = 0; k < NC; k++) scale[k] = scale[k] > 0 ? 1.0 / sqrt(scale[k] / cnt) : 1.0;
         std::vector<double> G((size_t)NC * NC, 0.0), rhs(NC, 0.0);
-        double x[2 + MLP_F];
-        for (long long i = 0; i < n; i++) {
-            if (!columns(i, x)) continue;
-            const double z = hl[i] - hf[i * MLP_F + 3];
-            for (int a = 0; a < NC; a++) {
-                const double xa = x[a] * scale[a];
-                rhs[a] += xa * z;
-                for (int b = 0; b <= a; b++) G[a * NC + b] += xa * x[b] * scale[b];
+        std::vector<double> sum((size_t)HOST_CHUNKS * NC * (NC + 1), 0.0);
+        host_chunks(n, [&](int q, long long b0, long long e0) {
+            double x[2 + MLP_F], t[(2 + MLP_F) * (3 + MLP_F)] = {};
+            for (long long i = b0; i < e0; i++) {
+                if (!columns(i, x)) continue;
+                const double z = hl[i] - hf[i * MLP_F + 3];
+                for (int a = 0; a < NC; a++) {
+                    const double xa = x[a] * scale[a];
+                    t[NC * NC + a] += xa * z;
+                    for (int b = 0; b <= a; b++) t[a * NC + b] += xa * x[b] * scale[b];
+                }
             }
+            std::copy(t, t + NC * (NC + 1), sum.begin() + (size_t)q * NC * (NC + 1));
+        });
+        for (int q = 0; q < HOST_CHUNKS; q++) {
+            const double* t = sum.data() + (size_t)q * NC * (NC + 1);
+            for (int a = 0; a < NC * NC; a++) G[a] += t[a];
+            for (int a = 0; a < NC; a++) rhs[a] += t[NC * NC + a];
         }
         for (int a = 0; a < NC; a++) {
             G[a * NC + a] += 1e-9 * cnt;  // ridge: keeps collinear columns solvable
@@ -2215,14 +2288,22 @@ extern "C" fmm_status fmm_mlp_train(fmm_ctx* c, const float* feats, const float*
         }
         if (ok) {
             for (int a = 0; a < NC; a++) coef[a] = coef[a] / G[a * NC + a] * scale[a];
+            std::vector<std::vector<float>> rq(HOST_CHUNKS);
+            for (int q = 0; q < HOST_CHUNKS; q++) rq[q].resize((size_t)(n * (q + 1) / HOST_CHUNKS - n * q / HOST_CHUNKS));
+            host_chunks(n, [&](int q, long long b0, long long e0) {
+                double x[2 + MLP_F];
+                size_t m = 0;
+                for (long long i = b0; i < e0; i++) {
+                    if (!columns(i, x)) continue;
+                    double y = hf[i * MLP_F + 3];
+                    for (int a = 0; a < NC; a++) y += coef[a] * x[a];
+                    rq[q][m++] = (float)(pred[i] - y);
+                }
+                rq[q].resize(m);
+            });
             std::vector<float> r;
             r.reserve((size_t)cnt);
-            for (long long i = 0; i < n; i++) {
-                if (!columns(i, x)) continue;
-                double y = hf[i * MLP_F + 3];
-                for (int a = 0; a < NC; a++) y += coef[a] * x[a];
-                r.push_back((float)(pred[i] - y));
-            }
+            for (const std::vector<float>& v : rq) r.insert(r.end(), v.begin(), v.end());
             const size_t klo = r.size() / 2000, khi = r.size() - 1 - r.size() / 2000;
             std::nth_element(r.begin(), r.begin() + klo, r.end());
             const float rlo = r[klo];
