@@ -400,70 +400,117 @@ def gen_pc():
     return L
 
 
+# Factors of the record as the particle-cell kernel stages it: the powers and binomials of the radial
+# factors go into the moments once per staged cell instead of into every pair (see gen_pc2).
+PC_SCALE = [Fraction(1)] + [Fraction(3)] * 6 + [Fraction(15, 2)] * 10 + [Fraction(35, 2)] * 15 + \
+           [Fraction(-1, 2)] + [Fraction(-3, 2)] * 3 + [Fraction(-15, 2)] * 6 + [Fraction(3, 8)] + [Fraction(0)]
+assert len(PC_SCALE) == NREC
+
+
+def gen_pc_scale():
+    L = ["/* factors of the record as fmm_pc_body2 takes it, by slot */",
+         "#define FMM_PC_SCALE {" + ", ".join(lit(v) for v in PC_SCALE) + "}"]
+    return L
+
+
 def gen_pc2():
-    """gen_pc for two sinks at once (FP32x2): the same field of one record at r0 and r1, as
-    float2 lanes.  Record values and constants are shared by both sinks; each multiply-add of the
-    scalar body becomes one __ffma2_rn, so a pair of sinks costs the FP32 instructions of one.
-    The potential is summed with the opposite sign (phip += ..., phi = -phip), so no negation is
-    issued per pair."""
+    """gen_pc for two sinks at once (FP32x2): the field of one record at r0 and r1, as float2 lanes.
+    Record values and constants are shared by both sinks, and each multiply-add is one __ffma2_rn.
+
+    With the record S scaled by PC_SCALE and Q the six products of q (off-diagonal ones doubled, so
+    that a contraction of a symmetric tensor with qq is six multiply-adds):
+      w = (S4:Q + Str4) . q,  W0 = w.q,  h = Str4:Q        (= 35/2 A1 - 15/2 T1, and -15/2 T0)
+      z = S3:Q + Str3,        z0 = z.q,  g = Str3.q        (= 15/2 B1 - 3/2 trM3, and -3/2 u0)
+      c = S2.q,               c0 = c.q                     (= 3 C1)
+    and, from the p, s and v of gen_pc (St2 = -t2/2, Stt4 = 3/8 tt4),
+      p2 = c0/2 + St2        s2 = -5/2 c0 - 3 St2
+      p3 = (z0 + 2 g)/3      s3 = -(7 z0 + 8 g)/3           v = c + ir (z + ir w)
+      p4 = (W0 + h)/4 + Stt4 s4 = -9/4 W0 - 5/4 h - 5 Stt4
+    Contracting with qq at once and adding the traces to the tensors before the last contraction
+    leaves 137 FP32x2 instructions of the 168 that one contraction per factor and separate trace
+    vectors take.  The potential is summed with the opposite sign (phip += ..., phi = -phip), so no
+    negation is issued per pair."""
     f2 = lambda x: f"make_float2({x}, {x})"
-    L = ["/* particle-cell for two sinks (FP32x2 lanes): field of the record R at r0 and r1; phip sums -phi */",
-         "__device__ __forceinline__ void fmm_pc_acc2(const float* __restrict__ R, float2 rx, float2 ry, float2 rz,",
-         "                                            float2 eps2, float2& ax, float2& ay, float2& az, float2& phip)",
+    fma = lambda x, y, z: f"__ffma2_rn({x}, {y}, {z})"
+    mul = lambda x, y: f"__fmul2_rn({x}, {y})"
+    L = ["/* particle-cell for two sinks (FP32x2 lanes): field at r0 and r1 of the record S scaled by",
+         "   FMM_PC_SCALE; phip sums -phi */",
+         "__device__ __forceinline__ void fmm_pc_body2(const float* __restrict__ S, float2 rx, float2 ry, float2 rz,",
+         "                                             float2 eps2, float2& ax, float2& ay, float2& az, float2& phip)",
          "{",
          "    const float2 r2 = __ffma2_rn(rx, rx, __ffma2_rn(ry, ry, __ffma2_rn(rz, rz, eps2)));",
          "    const float2 ir = make_float2(fmm_rsqrt(r2.x), fmm_rsqrt(r2.y));",
          "    const float2 qx = __fmul2_rn(rx, ir), qy = __fmul2_rn(ry, ir), qz = __fmul2_rn(rz, ir);",
-         "    const float2 ir2 = __fmul2_rn(ir, ir);"]
+         "    const float2 ir2 = __fmul2_rn(ir, ir);",
+         "    const float2 dx = __fadd2_rn(qx, qx), dy = __fadd2_rn(qy, qy);"]
     q = ["qx", "qy", "qz"]
+    two = [n for n in MI if sum(n) == 2]
+    Q = {}
+    for n in two:
+        i = [a for a in range(3) for _ in range(n[a])]
+        Q[n] = f"Q{n[0]}{n[1]}{n[2]}"
+        L.append(f"    const float2 {Q[n]} = " + (mul(q[i[0]], q[i[0]]) if i[0] == i[1] else mul("d" + "xyz"[i[0]], q[i[1]])) + ";")
 
-    def contract(rank, name, load, scalar):
-        lines, out = [], {}
-        for m in mindices(rank - 1):
-            if sum(m) != rank - 1:
-                continue
-            ops = [load(add(m, E[a])) for a in range(3)]
-            if scalar:
-                ops = [f2(o) for o in ops]
-            v = f"{name}{m[0]}{m[1]}{m[2]}"
-            lines.append(f"    const float2 {v} = __ffma2_rn({ops[2]}, {q[2]}, __ffma2_rn({ops[1]}, {q[1]}, "
-                         f"__fmul2_rn({ops[0]}, {q[0]})));")
-            out[m] = v
-        return lines, out
+    def against_qq(v, load, start):
+        """v = start + sum over the six products of load(n) Q[n]"""
+        e = start
+        for n in reversed(two):
+            e = mul(f2(load(n)), Q[n]) if e is None else fma(f2(load(n)), Q[n], e)
+        L.append(f"    const float2 {v} = {e};")
 
-    rec = lambda n: f"R[{MSLOT[n]}]"
-    l, A3 = contract(4, "A3_", rec, True); L += l
-    l, A2 = contract(3, "A2_", lambda n: A3[n], False); L += l
-    l, A1 = contract(2, "A1_", lambda n: A2[n], False); L += l
-    l, A0 = contract(1, "A0_", lambda n: A1[n], False); L += l
-    l, B2 = contract(3, "B2_", rec, True); L += l
-    l, B1 = contract(2, "B1_", lambda n: B2[n], False); L += l
-    l, B0 = contract(1, "B0_", lambda n: B1[n], False); L += l
-    l, C1 = contract(2, "C1_", rec, True); L += l
-    l, C0 = contract(1, "C0_", lambda n: C1[n], False); L += l
-    l, T1 = contract(2, "T1_", lambda n: f"R[{TR4[n]}]", True); L += l
-    l, T0 = contract(1, "T0_", lambda n: T1[n], False); L += l
-    l, U0 = contract(1, "U0_", lambda n: f"R[{TR3[n.index(1)]}]", True); L += l
-    a0, b0, c0, t0, u0 = A0[(0, 0, 0)], B0[(0, 0, 0)], C0[(0, 0, 0)], T0[(0, 0, 0)], U0[(0, 0, 0)]
-    t2, tt4, M = f"R[{TR2}]", f"R[{TT4}]", "R[0]"
+    def dot(v, x):
+        L.append(f"    const float2 {v} = {fma(x[2], q[2], fma(x[1], q[1], mul(x[0], q[0])))};")
+
+    slot = lambda n: f"S[{MSLOT[n]}]"
+    W = {}
+    for m in two:
+        W[m] = f"W{m[0]}{m[1]}{m[2]}"
+        against_qq(W[m], lambda n, m=m: slot(add(m, n)), f2(f"S[{TR4[m]}]"))
+    for a in range(3):
+        dot(f"w{'xyz'[a]}", [W[add(E[a], E[b])] for b in range(3)])
+    dot("W0", ["wx", "wy", "wz"])
+    against_qq("h", lambda n: f"S[{TR4[n]}]", None)
+    for a in range(3):
+        against_qq(f"z{'xyz'[a]}", lambda n, a=a: slot(add(E[a], n)), f2(f"S[{TR3[a]}]"))
+    dot("z0", ["zx", "zy", "zz"])
+    dot("g", [f2(f"S[{TR3[a]}]") for a in range(3)])
+    for a in range(3):
+        dot(f"c{'xyz'[a]}", [f2(slot(add(E[a], E[b]))) for b in range(3)])
+    dot("c0", ["cx", "cy", "cz"])
+    t2, tt4, M = f"S[{TR2}]", f"S[{TT4}]", "S[0]"
+    k = lambda v: f2(lit(v))
+    F = Fraction
     L += [
-        f"    const float2 p2 = __ffma2_rn({f2('1.5f')}, {c0}, {f2(f'-0.5f * {t2}')});",
-        f"    const float2 p3 = __ffma2_rn({f2('2.5f')}, {b0}, __fmul2_rn({f2('-1.5f')}, {u0}));",
-        f"    const float2 p4 = __ffma2_rn({f2('4.375f')}, {a0}, __ffma2_rn({f2('-3.75f')}, {t0}, {f2(f'0.375f * {tt4}')}));",
-        f"    const float2 s2 = __ffma2_rn({f2('-7.5f')}, {c0}, {f2(f'1.5f * {t2}')});",
-        f"    const float2 s3 = __ffma2_rn({f2('-17.5f')}, {b0}, __fmul2_rn({f2('7.5f')}, {u0}));",
-        f"    const float2 s4 = __ffma2_rn({f2('-39.375f')}, {a0}, __ffma2_rn({f2('26.25f')}, {t0}, {f2(f'-1.875f * {tt4}')}));",
-        f"    const float2 S = __ffma2_rn(ir2, __ffma2_rn(ir, __ffma2_rn(ir, s4, s3), s2), {f2(f'-{M}')});",
-        f"    phip = __ffma2_rn(ir, __ffma2_rn(ir2, __ffma2_rn(ir, __ffma2_rn(ir, p4, p3), p2), {f2(M)}), phip);",
+        f"    const float2 p2 = {fma(k(F(1, 2)), 'c0', f2(t2))};",
+        f"    const float2 p3 = {fma(k(F(1, 3)), 'z0', mul(k(F(2, 3)), 'g'))};",
+        f"    const float2 p4 = {fma(k(F(1, 4)), 'W0', fma(k(F(1, 4)), 'h', f2(tt4)))};",
+        f"    const float2 s2 = {fma(k(F(-5, 2)), 'c0', f2(f'-3.0f * {t2}'))};",
+        f"    const float2 s3 = {fma(k(F(-7, 3)), 'z0', mul(k(F(-8, 3)), 'g'))};",
+        f"    const float2 s4 = {fma(k(F(-9, 4)), 'W0', fma(k(F(-5, 4)), 'h', f2(f'-5.0f * {tt4}')))};",
+        f"    const float2 R = {fma('ir2', fma('ir', fma('ir', 's4', 's3'), 's2'), f2(f'-{M}'))};",
+        f"    phip = {fma('ir', fma('ir2', fma('ir', fma('ir', 'p4', 'p3'), 'p2'), f2(M)), 'phip')};",
     ]
-    for a, c in enumerate("xyz"):
-        m = E[a]
-        L.append(f"    const float2 w{c} = __ffma2_rn({f2('17.5f')}, {A1[m]}, __fmul2_rn({f2('-7.5f')}, {T1[m]}));")
-        L.append(f"    const float2 v{c} = __ffma2_rn({f2('3.0f')}, {C1[m]}, __fmul2_rn(ir, __ffma2_rn(ir, w{c}, "
-                 f"__ffma2_rn({f2('7.5f')}, {B1[m]}, {f2(f'-1.5f * R[{TR3[a]}]')}))));")
-        L.append(f"    a{c} = __ffma2_rn(ir2, __ffma2_rn(S, q{c}, __fmul2_rn(ir2, v{c})), a{c});")
+    for c in "xyz":
+        L.append(f"    const float2 v{c} = {fma('ir', fma('ir', f'w{c}', f'z{c}'), f'c{c}')};")
+        L.append(f"    a{c} = {fma('ir2', fma('R', f'q{c}', mul('ir2', f'v{c}')), f'a{c}')};")
     L.append("}")
+    L.append("")
+    L += ["/* the same from a record as the tree holds it (44 floats) */",
+          "__device__ __forceinline__ void fmm_pc_acc2(const float* __restrict__ R, float2 rx, float2 ry, float2 rz,",
+          "                                            float2 eps2, float2& ax, float2& ay, float2& az, float2& phip)",
+          "{",
+          "    const float f[FMM_NREC] = FMM_PC_SCALE;",
+          "    float S[FMM_NREC];",
+          "    for (int i = 0; i < FMM_NREC; i++) S[i] = f[i] * R[i];",
+          "    fmm_pc_body2(S, rx, ry, rz, eps2, ax, ay, az, phip);",
+          "}"]
     return L
+
+
+def count_flops2(lines):
+    """FP32 flops per sink of generated FP32x2 code (a multiply-add is 2)."""
+    body = "\n".join(lines[:lines.index("}")])
+    return 2 * body.count("__ffma2_rn(") + body.count("__fmul2_rn(") + body.count("__fadd2_rn(")
 
 
 def count_flops(lines):
@@ -488,7 +535,8 @@ def main():
     parts = {
         "green": gen_green_scaled(), "p2m": gen_p2m(), "m2m": gen_m2m(), "traces": gen_traces(),
         "norms": gen_norms(),
-        "m2l": gen_m2l(), "p2l": gen_p2l(), "l2l": gen_l2l(), "l2p": gen_l2p(), "pc": gen_pc(), "pc2": gen_pc2(),
+        "m2l": gen_m2l(), "p2l": gen_p2l(), "l2l": gen_l2l(), "l2p": gen_l2p(), "pc": gen_pc(), "pc_scale": gen_pc_scale(),
+        "pc2": gen_pc2(),
     }
     out = ["// GENERATED by gen_expansions.py -- do not edit by hand.",
            "// Straight-line FP32 expansion operators for the Plummer-softened Green's function,",
@@ -522,10 +570,11 @@ def main():
     for k, v in parts.items():
         out += v
         out.append("")
-    flops = {k: count_flops(v) for k, v in parts.items() if k != "pc2"}  # pc2: the pc arithmetic, paired
+    flops = {k: count_flops(v) for k, v in parts.items() if k not in ("pc2", "pc_scale")}
+    flops["pc2"] = count_flops2(parts["pc2"])
     out.append("/* FP32 flops of the generated bodies (fmaf = 2): " +
                ", ".join(f"{k} {v}" for k, v in flops.items()) + " */")
-    out.append(f"#define FMM_FLOPS_PC {flops['pc']}")
+    out.append(f"#define FMM_FLOPS_PC {flops['pc2']}")
     with open(os.path.join(here, "expansions.cuh"), "w") as f:
         f.write("\n".join(out) + "\n")
     print(flops)

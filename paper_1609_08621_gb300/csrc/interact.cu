@@ -32,8 +32,8 @@
 // by adding back the identically computed value.  Source particles are staged per warp in
 // shared memory (32 list entries at a time, <= 16 particles each).
 // PC: the order-4 moment record of each source cell evaluated at u_i - z_s
-// (fmm_pc_acc2: the trace form of fmm_pc_acc for two sinks).  Records of 32 cells are staged
-// per warp in shared memory.
+// (fmm_pc_body2, two sinks at once).  Records of 32 cells, scaled for it, are staged per warp in shared
+// memory.
 // L2P: the group's order-5 local coefficients evaluated at u_i.
 #include <algorithm>
 #include <atomic>
@@ -335,6 +335,8 @@ __device__ __forceinline__ int pc_pass_slots(int rem)
     return rem > 56 ? 64 : rem > 24 ? 32 : rem > 8 ? 16 : 8;
 }
 
+__constant__ float c_pc_scale[FMM_NREC] = FMM_PC_SCALE;
+
 // PC for one work item: each pass sweeps every staged chunk of cell records.  The sinks' offsets
 // (U, by slot) and each lane's running sums per pass (A: two float4 per lane and pass) stay in
 // shared memory between chunks, so one copy of the particle-cell body serves every pass.  Cell
@@ -345,7 +347,8 @@ __device__ __forceinline__ void pc_item(const Group& G, int nact, const int* __r
                                         const int* __restrict__ bucket_of, const int* __restrict__ bucket_cell,
                                         const float4* __restrict__ off, const float4* __restrict__ rec4,
                                         float4* __restrict__ part, float4* R4, float4* Zxy, float2* Zz, int* ids,
-                                        float4* U, float4* A, float eps2, int lane, int csize, int ib, int R)
+                                        float4* U, float4* A, const float4* F4, float eps2, int lane, int csize,
+                                        int ib, int R)
 {
     for (int i = lane; i < FMM_GMAX; i += 32) {
         float ux = 0.f, uy = 0.f, uz = 0.f, m;
@@ -385,7 +388,8 @@ __device__ __forceinline__ void pc_item(const Group& G, int nact, const int* __r
         const int nv = ne * (FMM_NREC / 4);
         for (int v = lane; v < nv; v += 32) {
             const int cl = v / (FMM_NREC / 4), q = v - cl * (FMM_NREC / 4);
-            R4[v] = rec4[(long long)ids[cl] * (FMM_NREC / 4) + q];
+            const float4 r = rec4[(long long)ids[cl] * (FMM_NREC / 4) + q], f = F4[q];
+            R4[v] = make_float4(r.x * f.x, r.y * f.y, r.z * f.z, r.w * f.w);
         }
         __syncwarp();
         for (int p = 0, base = 0; p < npass; p++) {
@@ -397,7 +401,7 @@ __device__ __forceinline__ void pc_item(const Group& G, int nact, const int* __r
             for (int j = split; j < ne; j += Q) {
                 const float4 zxy = Zxy[j];
                 const float2 zz = Zz[j];
-                fmm_pc_acc2(reinterpret_cast<const float*>(&R4[j * (FMM_NREC / 4)]),
+                fmm_pc_body2(reinterpret_cast<const float*>(&R4[j * (FMM_NREC / 4)]),
                             __fadd2_rn(ux, make_float2(zxy.x, zxy.y)), __fadd2_rn(uy, make_float2(zxy.z, zxy.w)),
                             __fadd2_rn(uz, zz), e2, bx, by, bz, bp);
             }
@@ -454,9 +458,12 @@ __global__ void __launch_bounds__(ITHREADS, 4) k_pc(const Group* __restrict__ gr
     __shared__ float2 Zzs[IW][PC_CHUNK];
     __shared__ int idss[IW][PC_CHUNK];
     __shared__ float4 Us[IW][FMM_GMAX], As[IW][PC_PMAX * 32 * 2];
+    __shared__ float4 F4[FMM_NREC / 4];  // the staged records' factors
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const float4* rec4 = reinterpret_cast<const float4*>(rec);
     if (fmm_overflowed(ctr)) return;
+    if (threadIdx.x < FMM_NREC) reinterpret_cast<float*>(F4)[threadIdx.x] = c_pc_scale[threadIdx.x];
+    __syncthreads();
     const unsigned long long n_items =
         min((unsigned long long)*(volatile unsigned int*)&ctr->n_item_pc, (unsigned long long)cap_items);
     unsigned long long pairs = 0;
@@ -471,7 +478,7 @@ __global__ void __launch_bounds__(ITHREADS, 4) k_pc(const Group* __restrict__ gr
         const float4 hk = cen[2 * G.cell], lk = cen[2 * G.cell + 1];
         const int n = cnact[G.cell];  // active sinks of the group
         pc_item(G, n, act, k, hk, lk, pc, cen, bucket_of, bucket_cell, off, rec4, part_pc + i * FMM_GMAX, R4s[wl], Zs[wl],
-                Zzs[wl], idss[wl], Us[wl], As[wl], eps2, lane, csize, ib, R);
+                Zzs[wl], idss[wl], Us[wl], As[wl], F4, eps2, lane, csize, ib, R);
         if (lane == 0) {
             const int nc = min(csize, G.pc_len - k * csize);
             pairs += (unsigned long long)cnact[G.cell] * (unsigned long long)nc;
