@@ -828,7 +828,7 @@ static fmm_status walk_levels(fmm_ctx* c, WalkArgs& a, int levels)
         }
         const LocalGrids g = fmm_local_grids(w, prev ? c->prev_cc_len : -1, prev ? c->prev_cp_len : -1, -1);
         CK(fmm_launch_local_level(t, w, c->ctr, a.eps2, -1, levels, g, s));
-        c->launches += 2 + levels;
+        c->launches += 2 + (int)fmm_ceil_div(levels, FMM_LOCAL_STEP);
     } else {
         for (int L = 0; L < levels; L++) {
             a.level = L;
@@ -838,7 +838,7 @@ static fmm_status walk_levels(fmm_ctx* c, WalkArgs& a, int levels)
             CK(cudaStreamWaitEvent(c->loc_stream, c->loc_fork, 0));
             const LocalGrids g = fmm_local_grids(w, c->prev_cc[L], c->prev_cp[L], c->prev_front[L]);
             CK(fmm_launch_local_level(t, w, c->ctr, a.eps2, L, levels, g, c->loc_stream));
-            c->launches += 1 + 3;
+            c->launches += 1 + 2 + (L % FMM_LOCAL_STEP == 0 ? 1 : 0);
         }
         CK(cudaEventRecord(c->loc_join, c->loc_stream));
         CK(cudaStreamWaitEvent(s, c->loc_join, 0));

@@ -112,11 +112,13 @@ struct __align__(16) Group {
     int pp_src;  // source particles in the PP list
     unsigned long long pp_off, pc_off;
     int pp_len, pc_len;
+    int level;   // walk level of the cell
 };
 
 #define FMM_LIST_CHUNK 64  // default list entries per PP / PC work item
 #define FMM_LOCAL_RANGE 512  // local entries per warp range of the own-expansion kernel
 #define FMM_GMAX 64       // sink slots per group
+#define FMM_LOCAL_STEP 4  // walk levels between those whose cells' local expansions are evaluated
 #define FMM_MAX_LEVELS 192  // walk levels: tree depth + 1 (63 key bits + 31 position bits at most)
 
 // Device-side counters and status, one per context.

@@ -21,8 +21,8 @@
 //
 // The local expansion of a walked cell is L_k = L2L(L_parent) + sum of M2L (CC) and P2L
 // (CP) terms.  A level's local lists are complete when its walk kernel ends, so a large walk runs
-// their M2L and P2L terms and the level's top-down pass on a side stream while the walk goes on
-// below; a small one runs them after its last level.
+// their M2L and P2L terms and the top-down passes on a side stream while the walk goes on below; a
+// small one runs them after its last level.
 #include <limits.h>
 
 #include <algorithm>
@@ -509,6 +509,7 @@ __device__ __forceinline__ void walk_sinks(const WalkIO& w, const unsigned long 
                 g.pc_off = co;
                 g.pp_len = npp;
                 g.pc_len = nx;
+                g.level = w.level;
                 w.groups[gi] = g;
             }
         } else {
@@ -667,16 +668,22 @@ __global__ void __launch_bounds__(LOCAL_THREADS, FMM_LOCAL_MINB) k_local_flat(
         const long long r1 = local_boundary(start + (r + 1) * LF_ENTRIES, total, cc_sink, lcc_off, lcc_len);
         float carry0 = 0.0f, carry1 = 0.0f;
         int carry_sink = -1;
+        // entries and sinks are read a chunk ahead: of a chunk's two dependent rounds of loads (they, then
+        // the centres and records) one passes behind the chunk before (M2L of a 384^3 box -7%)
+        unsigned int e_next = r0 + lane < r1 ? cc[r0 + lane] : 0u;
+        int sink_next = r0 + lane < r1 ? cc_sink[r0 + lane] : -1;
         for (long long base = r0; base < r1; base += 32) {
             const long long idx = base + lane;
             const bool valid = idx < r1;
-            int sink = -1;
+            const unsigned int e = e_next;
+            const int sink = sink_next;
+            e_next = idx + 32 < r1 ? cc[idx + 32] : 0u;
+            sink_next = idx + 32 < r1 ? cc_sink[idx + 32] : -1;
             float acc[FMM_NL];
 #pragma unroll
             for (int i = 0; i < FMM_NL; i++) acc[i] = 0.0f;
             if (valid) {
-                sink = cc_sink[idx];
-                local_entry<KIND>(cc[idx], cen[2 * sink], cen[2 * sink + 1], cen, posf, plo, rec, eps2, ib, R, acc);
+                local_entry<KIND>(e, cen[2 * sink], cen[2 * sink + 1], cen, posf, plo, rec, eps2, ib, R, acc);
                 nent++;
             }
 #pragma unroll
@@ -720,59 +727,166 @@ __global__ void __launch_bounds__(LOCAL_THREADS, FMM_LOCAL_MINB) k_local_flat(
     if (lane == 0 && nent) atomicAdd(KIND == 0 ? &ctr->n_cc : &ctr->n_cp, (unsigned long long)nent);
 }
 
-// The local expansion of every walked cell about its centre of mass, top-down one level per
-// launch: L(c) = L2L(L(parent), com(c) - com(parent)) + L_own(c), with L_own the sum of c's own
-// M2L and P2L terms (zero for a cell with empty lists) and a level-0 cell taking its own terms
-// only.  Written in place over L_own.  A local expansion is a polynomial of degree 5, so the chain
-// of re-expansions equals re-expanding every ancestor's own terms to the cell directly.  One
-// thread per cell.
+// The local expansion of a walked cell about its centre of mass, L(c) = L2L(L(parent), com(c) -
+// com(parent)) + L_own(c), with L_own the sum of c's own M2L and P2L terms (zero for a cell with empty
+// lists) and a level-0 cell taking its own terms only.  A local expansion is a polynomial of degree 5,
+// so the chain of re-expansions equals re-expanding every ancestor's own terms to the cell directly.
+//
+// Only groups need theirs, so not every level waits for the one above: every LD_STEP-th level (an
+// anchor level) is evaluated in place over its own terms, one launch each, and every group walks from
+// the last anchor above it, as an anchor does from the anchor before: at most LD_STEP re-expansions,
+// of which siblings repeat some.  The value of a cell is formed by the same operations whatever the
+// step.  Walk phase by step (128^3 NFW box / 384^3 box / 4096 particles): 1: 2.91 / 47.1 ms, 4: 2.77 /
+// 46.7 / 0.313, 6: 2.79 / 46.8 / 0.310.
+//
+// A warp takes a cell, two coefficients per lane, and shifts along one axis after the other:
+// sum_j t^j/j! L_(k + j e), the exact Taylor shift of a polynomial, about 100 instructions instead of
+// the 1095 flops of the shift in all three at once by one thread.  A launch is bound by its chain of
+// dependent loads and launch overhead.  One launch per level with a thread per cell took 441 us on the
+// 128^3 NFW box (36 levels), 348 us on a 63^3 one, 142 us on a 4096-particle box; the walk phase went
+// from 3.03 to 2.83 ms, 1.21 to 0.97 and 0.37 to 0.32 with this.
 #define LD_THREADS 128
-__global__ void __launch_bounds__(LD_THREADS) k_local_down(int level, const int* __restrict__ wcells, long long cap,
-                                                          const int* __restrict__ cparent,
-                                                          const int* __restrict__ lcc_len,
-                                                          const int* __restrict__ lcp_len,
-                                                          const Com4* __restrict__ com, float* __restrict__ L,
-                                                          const DevCounters* __restrict__ ctr)
+#define LD_STEP FMM_LOCAL_STEP
+
+// storage index of the coefficient (a, b, c) of order o = a + b + c, m = b + c (gen_expansions.py: order,
+// then a descending, then b descending)
+__device__ __forceinline__ int local_index(int o, int m, int c) { return o * (o + 1) * (o + 2) / 6 + m * (m + 1) / 2 + c; }
+
+// For coefficient q, per axis, the storage indices of k + j e for j = 1..5, six bits each; FMM_NL (a zero)
+// past order 5
+__device__ __forceinline__ void local_shift_index(int q, unsigned int idx[3])
 {
-    if (fmm_overflowed(ctr)) return;
-    const long long b0 = min((long long)ctr->lv_base[level], cap);
-    const long long b1 = min((long long)ctr->lv_base[level + 1], cap);
-    for (long long i = b0 + (long long)blockIdx.x * blockDim.x + threadIdx.x; i < b1;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int c = wcells[i];
-        float* Lc = L + (long long)c * FMM_NL;
-        float acc[FMM_NL];
-        if (lcc_len[c] > 0 || lcp_len[c] > 0) {
+    idx[0] = idx[1] = idx[2] = 0u;
+    int o = 0, m = 0;
+    while (o < 5 && q >= (o + 1) * (o + 2) * (o + 3) / 6) o++;
+    const int r = q - o * (o + 1) * (o + 2) / 6;
+    while (r >= (m + 1) * (m + 2) / 2) m++;
+    const int c = r - m * (m + 1) / 2;
 #pragma unroll
-            for (int q = 0; q < FMM_NL; q++) acc[q] = Lc[q];
-        } else {
-#pragma unroll
-            for (int q = 0; q < FMM_NL; q++) acc[q] = 0.0f;
-        }
-        if (level > 0) {
-            const int p = cparent[c];
-            const Com4 cc = com[c], cp = com[p];
-            float Lo[FMM_NL];
-            fmm_l2l(L + (long long)p * FMM_NL, __double2float_rn(cc.x - cp.x), __double2float_rn(cc.y - cp.y),
-                    __double2float_rn(cc.z - cp.z), Lo);
-#pragma unroll
-            for (int q = 0; q < FMM_NL; q++) acc[q] = Lo[q] + acc[q];
-        }
-#pragma unroll
-        for (int q = 0; q < FMM_NL; q++) Lc[q] = acc[q];
+    for (int j = 1; j <= 5; j++) {
+        const bool in = q < FMM_NL && o + j <= 5;
+        idx[0] |= (unsigned int)(in ? local_index(o + j, m, c) : FMM_NL) << (6 * (j - 1));
+        idx[1] |= (unsigned int)(in ? local_index(o + j, m + j, c) : FMM_NL) << (6 * (j - 1));
+        idx[2] |= (unsigned int)(in ? local_index(o + j, m + j, c + j) : FMM_NL) << (6 * (j - 1));
     }
 }
 
-// Each group's local expansion: its cell's, after the top-down pass.
-__global__ void k_local_groups(const Group* __restrict__ groups, const float* __restrict__ L, float* __restrict__ Lg,
-                               long long cap_groups, const DevCounters* __restrict__ ctr)
+// Coefficients lane and lane + 32 of the expansion of cell c from that of its ancestor `steps` levels up,
+// whose row of L is complete (its own terms only, for done = false); buf: two rows of FMM_NL + 1 values
+// of this warp.
+__device__ __forceinline__ void local_chain(int c, int steps, bool done, const int* __restrict__ cparent,
+                                            const int* __restrict__ lcc_len, const int* __restrict__ lcp_len,
+                                            const float4* __restrict__ cen, const float* L, float (*buf)[FMM_NL + 1],
+                                            const unsigned int i0[3], const unsigned int i1[3], int lane, float& v0, float& v1)
 {
+    const bool two = lane + 32 < FMM_NL;
+    // own terms and centres along the path, all loads in flight together
+    float w0[LD_STEP], w1[LD_STEP];
+    float4 h[LD_STEP + 1], l[LD_STEP + 1];
+    int x = c;
+#pragma unroll
+    for (int s = 0; s <= LD_STEP; s++) {
+        if (s > steps) break;
+        h[s] = cen[2 * x];
+        l[s] = cen[2 * x + 1];
+        const bool own = (done && s == steps) || lcc_len[x] > 0 || lcp_len[x] > 0;
+        const float* row = L + (long long)x * FMM_NL;
+        const float a = own ? row[lane] : 0.0f, b = own && two ? row[lane + 32] : 0.0f;
+        if (s == steps) {
+            v0 = a;
+            v1 = b;
+        } else {
+            w0[s] = a;
+            w1[s] = b;
+        }
+        if (s < steps) x = cparent[x];
+    }
+#pragma unroll
+    for (int s = LD_STEP - 1; s >= 0; s--) {
+        if (s >= steps) continue;
+        const float t[3] = {cen_diff(h[s].x, l[s].x, h[s + 1].x, l[s + 1].x),
+                            cen_diff(h[s].y, l[s].y, h[s + 1].y, l[s + 1].y),
+                            cen_diff(h[s].z, l[s].z, h[s + 1].z, l[s + 1].z)};
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            float* const row = buf[a & 1];
+            row[lane] = v0;
+            if (two) row[lane + 32] = v1;
+            __syncwarp();
+            float p = t[a];
+            const float inv[5] = {1.0f, 1.0f / 2.0f, 1.0f / 3.0f, 1.0f / 4.0f, 1.0f / 5.0f};
+#pragma unroll
+            for (int j = 0; j < 5; j++) {  // p = t^(j + 1) / (j + 1)!
+                v0 = fmaf(p, row[(i0[a] >> (6 * j)) & 63u], v0);
+                v1 = fmaf(p, row[(i1[a] >> (6 * j)) & 63u], v1);
+                if (j < 4) p *= t[a] * inv[j + 1];
+            }
+        }
+        v0 += w0[s];
+        v1 += w1[s];
+        __syncwarp();  // the first row is free again
+    }
+}
+
+// The cells of an anchor level, over their own terms.
+__global__ void __launch_bounds__(LD_THREADS) k_local_anchor(int level, const int* __restrict__ wcells, long long cap,
+                                                            const int* __restrict__ cparent,
+                                                            const int* __restrict__ lcc_len,
+                                                            const int* __restrict__ lcp_len,
+                                                            const float4* __restrict__ cen, float* L,
+                                                            const DevCounters* __restrict__ ctr)
+{
+    __shared__ float buf[LD_THREADS / 32][2][FMM_NL + 1];
+    if (fmm_overflowed(ctr)) return;
+    const long long b0 = min((long long)ctr->lv_base[level], cap);
+    const long long b1 = min((long long)ctr->lv_base[level + 1], cap);
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    if (b0 + gw >= b1) return;
+    unsigned int i0[3], i1[3];
+    local_shift_index(lane, i0);
+    local_shift_index(lane + 32, i1);
+    if (lane < 2) buf[wl][lane][FMM_NL] = 0.0f;
+    __syncwarp();
+    for (long long i = b0 + gw; i < b1; i += nw) {
+        const int c = wcells[i];
+        float v0, v1;
+        local_chain(c, level == 0 ? 0 : LD_STEP, level > 0, cparent, lcc_len, lcp_len, cen, L, buf[wl], i0, i1, lane, v0, v1);
+        float* row = L + (long long)c * FMM_NL;
+        row[lane] = v0;
+        if (lane + 32 < FMM_NL) row[lane + 32] = v1;
+    }
+}
+
+// Each group's local expansion, from the last anchor level at or above it.
+__global__ void __launch_bounds__(LD_THREADS) k_local_groups(const Group* __restrict__ groups,
+                                                            const int* __restrict__ cparent,
+                                                            const int* __restrict__ lcc_len,
+                                                            const int* __restrict__ lcp_len,
+                                                            const float4* __restrict__ cen, const float* L,
+                                                            float* __restrict__ Lg, long long cap_groups,
+                                                            const DevCounters* __restrict__ ctr)
+{
+    __shared__ float buf[LD_THREADS / 32][2][FMM_NL + 1];
     if (fmm_overflowed(ctr)) return;
     const long long ng = min((long long)*(volatile const unsigned long long*)&ctr->n_groups, cap_groups);
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < ng * FMM_NL;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long gi = i / FMM_NL;
-        Lg[i] = L[(long long)groups[gi].cell * FMM_NL + (i - gi * FMM_NL)];
+    const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    if (gw >= ng) return;
+    unsigned int i0[3], i1[3];
+    local_shift_index(lane, i0);
+    local_shift_index(lane + 32, i1);
+    if (lane < 2) buf[wl][lane][FMM_NL] = 0.0f;
+    __syncwarp();
+    for (long long gi = gw; gi < ng; gi += nw) {
+        const int c = groups[gi].cell, level = groups[gi].level;
+        float v0, v1;
+        local_chain(c, level % LD_STEP, true, cparent, lcc_len, lcp_len, cen, L, buf[wl], i0, i1, lane, v0, v1);
+        float* row = Lg + gi * FMM_NL;
+        row[lane] = v0;
+        if (lane + 32 < FMM_NL) row[lane + 32] = v1;
     }
 }
 
@@ -941,9 +1055,9 @@ cudaError_t fmm_launch_walk_level(DevTree& t, DevWalk& w, DevCounters* ctr, cons
     return cudaGetLastError();
 }
 
-// The local expansions of walk level `level` (-1: the whole lists, then every level's top-down
-// pass): its own M2L terms, then its P2L terms, then the top-down pass of its cells (which reads the
-// level above, done by an earlier call on the same stream).  The grids are the caller's: every
+// The local expansions of walk level `level` (-1: the whole lists, then every anchor level): its own M2L
+// terms, then its P2L terms, then, on an anchor level, its cells' expansions (which read the levels
+// above, done by earlier calls on the same stream).  The grids are the caller's: every
 // kernel takes its work with grid-stride loops, so any size gives the same result.
 cudaError_t fmm_launch_local_level(DevTree& t, DevWalk& w, DevCounters* ctr, float eps2, int level, int levels,
                                    const LocalGrids& g, cudaStream_t s)
@@ -954,8 +1068,9 @@ cudaError_t fmm_launch_local_level(DevTree& t, DevWalk& w, DevCounters* ctr, flo
                                                     t.plo, t.rec, t.L, w.cap_cp, eps2, t.per_ib, t.per_R, level, ctr);
     const int l0 = level < 0 ? 0 : level, l1 = level < 0 ? levels : level + 1;
     for (int l = l0; l < l1; l++)
-        k_local_down<<<g.down, LD_THREADS, 0, s>>>(l, w.wcells, w.cap_front, t.cparent, w.lcc_len, w.lcp_len, t.com,
-                                                   t.L, ctr);
+        if (l % LD_STEP == 0)
+            k_local_anchor<<<g.down, LD_THREADS, 0, s>>>(l, w.wcells, w.cap_front, t.cparent, w.lcc_len, w.lcp_len,
+                                                         t.cen, t.L, ctr);
     return cudaGetLastError();
 }
 
@@ -979,7 +1094,7 @@ LocalGrids fmm_local_grids(const DevWalk& w, long long n_cc, long long n_cp, lon
     g.cp = flat(n_cp);
     g.down = n_cells < 0 ? (unsigned)full_down
                          : (unsigned)std::max(std::min(floor, full_down),
-                                              std::min(full_down, fmm_ceil_div(n_cells * 5 / 4 + 1, LD_THREADS)));
+                                              std::min(full_down, fmm_ceil_div(n_cells * 5 / 4 + 1, LD_THREADS / 32)));
     return g;
 }
 
@@ -988,6 +1103,7 @@ cudaError_t fmm_launch_local_groups(DevWalk& w, DevTree& t, DevCounters* ctr, cu
     int sms = 152, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    k_local_groups<<<(unsigned)(sms * 8), 256, 0, s>>>(w.groups, t.L, w.Lg, w.cap_groups, ctr);
+    k_local_groups<<<(unsigned)(sms * 16), LD_THREADS, 0, s>>>(w.groups, t.cparent, w.lcc_len, w.lcp_len, t.cen, t.L, w.Lg,
+                                                             w.cap_groups, ctr);
     return cudaGetLastError();
 }
