@@ -556,10 +556,9 @@ static fmm_status build_tree(fmm_ctx* c, const double* pos, const float* mass, c
     CK(fmm_launch_keys(t, pos, mass, active, n, c->ctr, s, c->cur_ipos));
     if (nbox > 1) {
         CK(fmm_launch_box_sort(t, n, s));
-        c->launches += 8 * 5 + 1 + 2 * 5 + 1;
+        c->launches += 2;
     } else {
         CK(fmm_radix_sort(t, n, s));
-        c->launches += 8 * 5;
     }
     CK(fmm_launch_gather(t, n, c->ctr, s));
     CK(fmm_launch_radix_tree(t, n, bucket, s));
@@ -604,9 +603,9 @@ static fmm_status build_tree(fmm_ctx* c, const double* pos, const float* mass, c
         CK(fmm_launch_box_roots(t, s));
         c->launches += 1;
     }
-    // keys, gather, radix tree + keep, scan, cells, scan, bucket index, depth, bucket cells,
-    // upward, exact b_max (count, scan, expand, item order: count, scan, place; two passes, final)
-    c->launches += 1 + 1 + (n > 1 ? 2 : 1) + 3 + 1 + 3 + 1 + 1 + 2 + 13;
+    // keys, gather, radix tree + keep, cells, bucket index, depth, bucket cells, upward, exact b_max
+    // (count, expand, two passes, final); scans, sorts and the item order count themselves
+    c->launches += 1 + 1 + (n > 1 ? 2 : 1) + 1 + 1 + 1 + 2 + 5;
     t.depth = (int)c->ctr_h->depth;
     t.graded = t.grade_key != nullptr && n > 1;
     c->have_tree = true;
@@ -957,7 +956,7 @@ static fmm_status solve_eager(fmm_ctx* c, const double* pos, const float* mass, 
     cudaStream_t s = c->stream;
     c->have_solve = false;
     memset(&c->stats, 0, sizeof c->stats);
-    c->launches = 0;
+    c->launches = c->t.n_launches = 0;
     CK(cudaEventRecord(c->ev[0], s));
     st = build_tree(c, pos, mass, active, n, q.bucket, box_off, nbox);
     if (st != FMM_OK) return st;
@@ -1017,7 +1016,7 @@ static fmm_status interact_and_finish(fmm_ctx* c, const fmm_params& q, double ep
             w.cap_item_pc = need_pc;
         }
         CK(fmm_launch_items(c->t, w, c->ctr, ia.chunk, s));
-        c->launches += 3 + 2 * 3;
+        c->launches += 3;
         CK(fmm_launch_pp(c->t, c->w, c->ctr, ia, s));
         CK(cudaEventRecord(c->ev[3], s));
         CK(fmm_launch_pc(c->t, c->w, c->ctr, ia, s));
@@ -1062,7 +1061,7 @@ static fmm_status finish_stats(fmm_ctx* c, long long n)
     S.paper_flops = 53.0 * S.n_pp_pairs + 215.0 * S.n_pc_pairs + 479.0 * S.n_cc + 213.0 * S.n_cp;
     S.kernel_flops_pp = 19.0 * S.n_pp_pairs;
     S.kernel_flops_pc = (double)FMM_FLOPS_PC * S.n_pc_pairs;
-    S.n_launches = c->launches;
+    S.n_launches = c->launches + c->t.n_launches;
     S.n_learned = (long long)c->ctr_h->n_mlp;
     c->have_solve = true;
     return FMM_OK;
@@ -1082,7 +1081,7 @@ static fmm_status enqueue_graph_head(fmm_ctx* c, const double* pos, const float*
 {
     DevTree& t = c->t;
     cudaStream_t s = c->stream;
-    c->launches = 0;
+    c->launches = c->t.n_launches = 0;
     CK(cudaEventRecordWithFlags(c->ev[0], s, cudaEventRecordExternal));
     fmm_status st = set_boxes(c, n, box_off, nbox);
     if (st != FMM_OK) return st;
@@ -1092,16 +1091,15 @@ static fmm_status enqueue_graph_head(fmm_ctx* c, const double* pos, const float*
     CK(fmm_launch_keys(t, pos, mass, active, n, c->ctr, s, c->cur_ipos));
     if (nbox > 1) {
         CK(fmm_launch_box_sort(t, n, s));
-        c->launches += 8 * 5 + 1 + 2 * 5 + 1;
+        c->launches += 2;
     } else {
         CK(fmm_radix_sort(t, n, s));
-        c->launches += 8 * 5;
     }
     CK(fmm_launch_gather(t, n, c->ctr, s));
     CK(fmm_launch_radix_tree(t, n, q.bucket, s));
     CK(fmm_scan_exclusive(t.keep, t.keep, 2 * n - 1, c->totals, t, s));
     CK(cudaMemcpyAsync(c->totals_h, c->totals, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
-    c->launches += 1 + 1 + (n > 1 ? 2 : 1) + 3;
+    c->launches += 1 + 1 + (n > 1 ? 2 : 1);
     return FMM_OK;
 }
 
@@ -1125,7 +1123,7 @@ static fmm_status enqueue_graph_rest(fmm_ctx* c, long long n, const fmm_params& 
         CK(fmm_launch_box_roots(t, s));
         c->launches += 1;
     }
-    c->launches += 1 + 3 + 1 + 1 + 2 + 13;
+    c->launches += 1 + 1 + 1 + 2 + 5;
     CK(fmm_launch_nodes(t, q.theta, s));
     c->launches += 1;
     if (t.per_R > 0) {
@@ -1174,7 +1172,7 @@ static fmm_status enqueue_graph_rest(fmm_ctx* c, long long n, const fmm_params& 
     ia.accumulate = q.accumulate;
     ia.chunk = q.list_chunk ? q.list_chunk : FMM_LIST_CHUNK;
     CK(fmm_launch_items(t, w, c->ctr, ia.chunk, s));
-    c->launches += 3 + 2 * 3;
+    c->launches += 3;
     CK(fmm_launch_pp(t, w, c->ctr, ia, s));
     CK(cudaEventRecordWithFlags(c->ev[3], s, cudaEventRecordExternal));
     CK(fmm_launch_pc(t, w, c->ctr, ia, s));
@@ -1274,7 +1272,7 @@ static void capture_graph(fmm_ctx* c, const fmm_ctx::GraphKey& key, const double
     const int saved_launches = c->launches;
     cudaGraphExec_t head = capture_part(c, [&] { return enqueue_graph_head(c, pos, mass, active, n, q, box_off, nbox); });
     cudaGraphExec_t rest = head ? capture_part(c, [&] { return enqueue_graph_rest(c, n, q, acc, pot, nbox); }) : nullptr;
-    c->graph_launches = c->launches;  // both parts
+    c->graph_launches = c->launches + c->t.n_launches;  // both parts
     c->launches = saved_launches;
     if (!head || !rest) {
         if (head) cudaGraphExecDestroy(head);
@@ -1324,6 +1322,7 @@ static fmm_status replay_graph(fmm_ctx* c, long long n, int* outcome)
     memset(&c->stats, 0, sizeof c->stats);
     c->stats.n_active = (long long)h.n_active;
     c->launches = c->graph_launches;
+    t.n_launches = 0;
     st = finish_stats(c, n);
     if (st != FMM_OK) return st;
     c->graph_replays++;
@@ -1498,7 +1497,7 @@ static fmm_status select_subset(fmm_ctx* c, const double* pos, const double* vel
     CK(cudaMemcpyAsync(c->totals_h + 2, c->totals + 2, sizeof(unsigned int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     *m = (long long)c->totals_h[2];
-    c->launches += 4;
+    c->launches += 1;
     if (*m > 0) {
         CK(fmm_launch_subset_gather(c->d_flag, c->d_at, n, pos, vel, dt, mass, sinks, *m, c->d_pos, c->d_mass, c->d_act,
                                     c->d_idx, s));
@@ -1518,7 +1517,7 @@ extern "C" fmm_status fmm_set_fixed_sources(fmm_ctx* c, const double* pos, const
     FixedTree& f = c->fx;
     f.valid = false;
     c->have_solve = false;
-    c->launches = 0;
+    c->launches = c->t.n_launches = 0;
     long long m = 0;
     st = select_subset(c, pos, vel, dt, mass, rung, r_fixed, nullptr, nullptr, n, &m);
     if (st != FMM_OK) return st;
@@ -1590,7 +1589,7 @@ extern "C" fmm_status fmm_set_fixed_sources(fmm_ctx* c, const double* pos, const
     c->stats.n = m;
     c->stats.n_cells = f.n_cells;
     c->stats.n_buckets = f.n_buckets;
-    c->stats.n_launches = c->launches;
+    c->stats.n_launches = c->launches + c->t.n_launches;
     return FMM_OK;
 }
 
@@ -1621,7 +1620,7 @@ extern "C" fmm_status fmm_compute_forces_dual(fmm_ctx* c, const double* pos, con
     cudaStream_t s = c->stream;
     c->have_solve = false;
     memset(&c->stats, 0, sizeof c->stats);
-    c->launches = 0;
+    c->launches = c->t.n_launches = 0;
     CK(cudaEventRecord(c->ev[0], s));
     // the active tree: every particle outside the fixed set, at its current position
     long long na = 0;
@@ -2350,7 +2349,7 @@ extern "C" fmm_status fmm_mlp_audit(fmm_ctx* c, const double* pos, const float* 
         CK(alloc(&c->audit_pairs, max_pairs));
         c->audit_cap = max_pairs;
     }
-    c->launches = 0;
+    c->launches = c->t.n_launches = 0;
     st = build_tree(c, pos, mass, nullptr, n, q.bucket);
     if (st == FMM_OK) {
         cudaError_t e = fmm_launch_nodes(c->t, theta, s);

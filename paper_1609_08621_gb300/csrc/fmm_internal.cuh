@@ -251,6 +251,7 @@ struct DevTree {
     long long cap_scan_part = 0;
     unsigned int *hist = nullptr;
     long long cap_hist = 0;
+    int n_launches = 0;  // kernels launched by the scans and sorts of the current solve
 };
 
 __host__ __forceinline__ PeriodicArgs periodic_args(const DevTree& t)
@@ -327,7 +328,7 @@ long long fmm_sort_part_entries(long long n);
 cudaError_t fmm_sort_prepare();
 cudaError_t fmm_radix_sort_kv_scratch(unsigned long long* ka, unsigned long long* kb, unsigned int* va,
                                       unsigned int* vb, long long n, int passes, unsigned int* hist,
-                                      unsigned int* part, cudaStream_t s);
+                                      unsigned int* tot, int* launches, cudaStream_t s);
 
 // tree.cu
 // positions: pos (FP64 SoA) or, when ipos is given, 32-bit fixed-point coordinates x = u 2^-32

@@ -24,7 +24,7 @@ namespace {
 constexpr long long kMaxN = FMM_STATIC_ORDER_MAX_N;
 // scratch regions, each starting on a 256-byte boundary
 constexpr long long kHistCap = 256LL * (kMaxN / 1024);  // digit counts: 256 per tile of >= 1024 keys
-constexpr long long kPartCap = 4096;                     // partial sums of their scan
+constexpr long long kPartCap = 4096;                     // the digits' totals of each pass
 constexpr long long kOffKeyAlt = 0;
 constexpr long long kOffIdxAlt = kOffKeyAlt + 8 * kMaxN;
 constexpr long long kOffHist = kOffIdxAlt + 4 * kMaxN;
@@ -109,15 +109,16 @@ extern "C" fmm_status fmm_morton_order_static(const double* pos, long long n, un
     unsigned int* hist = reinterpret_cast<unsigned int*>(base + kOffHist);
     unsigned int* part = reinterpret_cast<unsigned int*>(base + kOffPart);
     unsigned int* status = reinterpret_cast<unsigned int*>(base + kOffStatus);
-    // the status word is the only scratch that must start at zero: the sort writes every digit
-    // count and partial sum it reads
+    // the status word is the only scratch that must start at zero: the sort clears the totals and
+    // writes every digit count that it reads
     e = cudaMemsetAsync(status, 0, sizeof(unsigned int), s);
     if (e != cudaSuccess) return report_cuda(e, "clearing the status word");
     k_order_keys<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(pos, n, keys, order, status);
     e = cudaGetLastError();
     if (e != cudaSuccess) return report_cuda(e, "key kernel");
     // 8 passes (an even number): the sorted keys and order end in the caller's buffers
-    e = fmm_radix_sort_kv_scratch(keys, key_alt, order, idx_alt, n, 8, hist, part, s);
+    int launches = 0;
+    e = fmm_radix_sort_kv_scratch(keys, key_alt, order, idx_alt, n, 8, hist, part, &launches, s);
     if (e != cudaSuccess) return report_cuda(e, "radix sort");
     unsigned int st_h = 0;
     e = cudaMemcpyAsync(&st_h, status, sizeof st_h, cudaMemcpyDeviceToHost, s);

@@ -489,7 +489,10 @@ long long fmm_bmax_items_bound(long long n, int depth, long long n_cells)
 // The passes take the items ordered by the particle they start at (counted per BM_CHUNK particles,
 // then placed): the warps in flight then read the same particles for the cells of every level
 // around them, from L2, instead of streaming all particles once per level.  Every item keeps its
-// index (its FP32 maximum is stored under it), and the maxima are order-independent.
+// index (its FP32 maximum is stored under it), and the maxima are order-independent.  While the
+// particles' positions fit L2 several times over (n <= BM_UNORDERED) the items keep the cells' order,
+// which saves six launches.
+#define BM_UNORDERED (1LL << 21)
 long long fmm_bmax_bins(long long n) { return fmm_ceil_div(n, BM_CHUNK) + 1; }
 
 __device__ __forceinline__ unsigned int bm_bin_of(long long i, const int* __restrict__ item,
@@ -642,7 +645,7 @@ __global__ void __launch_bounds__(256) k_bm_pass(const unsigned int* __restrict_
         float px = 0.0f, py = 0.0f, pz = 0.0f, thr = 0.0f;
         bool ok = false;
         if (ii < ni) {
-            i = order[ii];
+            i = order ? (long long)order[ii] : ii;
             // an item the expansion could not write (capacity overflow, reported to the host) is skipped
             c = item[i];
             if (c >= 0 && c < nc) {
@@ -737,7 +740,8 @@ cudaError_t fmm_launch_upward(DevTree& t, long long n, int bucket, DevCounters* 
     cudaError_t e = fmm_scan_exclusive(t.bm_cnt, t.bm_base, nc, &ctr->n_bm_items, t, s);
     if (e != cudaSuccess) return e;
     k_bm_expand<<<gb, TB, 0, s>>>(nc, t.bm_cnt, t.bm_base, t.bm_item, t.cap_bm_items, &ctr->overflow);
-    {
+    const bool ordered = n > BM_UNORDERED;
+    if (ordered) {
         const long long nbins = fmm_bmax_bins(n);
         const unsigned ob = (unsigned)std::max(1LL, std::min(fmm_ceil_div(t.cap_bm_items, TB), 152LL * 32));
         cudaMemsetAsync(t.bm_bin, 0, sizeof(unsigned int) * (size_t)nbins, s);
@@ -747,16 +751,18 @@ cudaError_t fmm_launch_upward(DevTree& t, long long n, int bucket, DevCounters* 
         if (e != cudaSuccess) return e;
         k_bm_place<<<ob, TB, 0, s>>>(t.bm_item, &ctr->n_bm_items, t.cap_bm_items, t.dcount, t.bm_base, t.cfirst,
                                       t.bm_binbase, t.bm_order);
+        t.n_launches += 2;
     }
+    const unsigned int* const order = ordered ? t.bm_order : nullptr;
     int sms = 152, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const long long want = fmm_ceil_div(t.cap_bm_items, 8);
     const unsigned pb = (unsigned)std::max(1LL, std::min(want, (long long)sms * 8));
-    k_bm_pass<1><<<pb, 256, 0, s>>>(t.bm_order, t.bm_item, &ctr->n_bm_items, t.cap_bm_items, t.dcount, t.bm_cnt, t.bm_base,
+    k_bm_pass<1><<<pb, 256, 0, s>>>(order, t.bm_item, &ctr->n_bm_items, t.cap_bm_items, t.dcount, t.bm_cnt, t.bm_base,
                                     t.cfirst, t.ccount,
                                     t.com, t.posf, t.sx, t.sy, t.sz, t.bm32, t.bm64, t.bm_imax);
-    k_bm_pass<2><<<pb, 256, 0, s>>>(t.bm_order, t.bm_item, &ctr->n_bm_items, t.cap_bm_items, t.dcount, t.bm_cnt, t.bm_base,
+    k_bm_pass<2><<<pb, 256, 0, s>>>(order, t.bm_item, &ctr->n_bm_items, t.cap_bm_items, t.dcount, t.bm_cnt, t.bm_base,
                                     t.cfirst, t.ccount,
                                     t.com, t.posf, t.sx, t.sy, t.sz, t.bm32, t.bm64, t.bm_imax);
     k_bm_final<<<gb, TB, 0, s>>>(t.dcount, t.cchild, t.bm64, t.bmax);
