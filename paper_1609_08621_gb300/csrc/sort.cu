@@ -168,15 +168,12 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const unsigned long long
     for (int i = tid; i < RS_WARPS * 256; i += RS_THREADS) c[i] = 0;
     __syncthreads();
     const long long t0 = (long long)blockIdx.x * RS_TILE + (long long)w * 32 * RS_ITEMS;
-    const unsigned int lt = fmm_lanemask_lt();
-#pragma unroll 4
+    // one count per key with shared-memory atomics into the warp's own counters (matching lanes first, as
+    // the scatter must to rank them, costs more than the conflicts it saves)
+#pragma unroll
     for (int r = 0; r < RS_ITEMS; r++) {
-        long long i = t0 + r * 32 + lane;
-        bool ok = i < n;
-        unsigned int d = ok ? (unsigned int)((kin[i] >> shift) & 255u) : 256u;
-        unsigned int peers = __match_any_sync(FMM_FULL_MASK, d);
-        if (ok && (peers & lt) == 0) c[w * 256 + d] += __popc(peers);
-        __syncwarp();
+        const long long i = t0 + r * 32 + lane;
+        if (i < n) atomicAdd(&c[w * 256 + (unsigned int)((kin[i] >> shift) & 255u)], 1u);
     }
     __syncthreads();
     unsigned int s = 0;
