@@ -940,8 +940,8 @@ static fmm_status run_walk(fmm_ctx* c, long long n, double eps, int bucket, int 
 }
 
 static fmm_status finish_stats(fmm_ctx* c, long long n);
-static fmm_status interact_and_finish(fmm_ctx* c, const fmm_params& q, double eps, float* acc, float* pot,
-                                      long long n_out, long long n_stats, const unsigned int* perm);
+static fmm_status interact_and_finish(fmm_ctx* c, const fmm_params& q, double eps, const unsigned char* active,
+                                      float* acc, float* pot, long long n_out, long long n_stats, const unsigned int* perm);
 
 static fmm_status solve_eager(fmm_ctx* c, const double* pos, const float* mass, const unsigned char* active, long long n,
                         double eps, double theta, float* acc, float* pot, const long long* box_off = nullptr,
@@ -981,14 +981,14 @@ static fmm_status solve_eager(fmm_ctx* c, const double* pos, const float* mass, 
     }
     st = run_walk(c, n, eps, q.bucket, q.group, q.criterion);
     if (st != FMM_OK) return st;
-    return interact_and_finish(c, q, eps, acc, pot, n, n, nullptr);
+    return interact_and_finish(c, q, eps, active, acc, pot, n, n, nullptr);
 }
 
 // After the walk: work items, PP, PC, and the sums plus local expansion written to acc/pot
 // (n_out particles long, in the order perm gives; NULL: the tree's own order); then the counters
 // and timing events are read back.
-static fmm_status interact_and_finish(fmm_ctx* c, const fmm_params& q, double eps, float* acc, float* pot,
-                                      long long n_out, long long n_stats, const unsigned int* perm)
+static fmm_status interact_and_finish(fmm_ctx* c, const fmm_params& q, double eps, const unsigned char* active,
+                                      float* acc, float* pot, long long n_out, long long n_stats, const unsigned int* perm)
 {
     cudaStream_t s = c->stream;
     fmm_status st;
@@ -1021,7 +1021,7 @@ static fmm_status interact_and_finish(fmm_ctx* c, const fmm_params& q, double ep
         CK(cudaEventRecord(c->ev[3], s));
         CK(fmm_launch_pc(c->t, c->w, c->ctr, ia, s));
         CK(cudaEventRecord(c->ev[4], s));
-        CK(fmm_launch_l2p_out(c->t, c->w, c->ctr, ia, acc, pot, n_out, s, perm));
+        CK(fmm_launch_l2p_out(c->t, c->w, c->ctr, ia, active, (long long)c->ctr_h->n_active, acc, pot, n_out, s, perm));
         c->launches += ((q.terms & 1) ? 1 : 0) + ((q.terms & 2) ? 1 : 0) + 1;
     } else {
         CK(cudaEventRecord(c->ev[3], s));
@@ -1103,7 +1103,8 @@ static fmm_status enqueue_graph_head(fmm_ctx* c, const double* pos, const float*
     return FMM_OK;
 }
 
-static fmm_status enqueue_graph_rest(fmm_ctx* c, long long n, const fmm_params& q, float* acc, float* pot, int nbox)
+static fmm_status enqueue_graph_rest(fmm_ctx* c, const unsigned char* active, long long n, const fmm_params& q,
+                                     float* acc, float* pot, int nbox)
 {
     DevTree& t = c->t;
     DevWalk& w = c->w;
@@ -1177,7 +1178,7 @@ static fmm_status enqueue_graph_rest(fmm_ctx* c, long long n, const fmm_params& 
     CK(cudaEventRecordWithFlags(c->ev[3], s, cudaEventRecordExternal));
     CK(fmm_launch_pc(t, w, c->ctr, ia, s));
     CK(cudaEventRecordWithFlags(c->ev[4], s, cudaEventRecordExternal));
-    CK(fmm_launch_l2p_out(t, w, c->ctr, ia, acc, pot, n, s));
+    CK(fmm_launch_l2p_out(t, w, c->ctr, ia, active, (long long)c->ctr_h->n_active, acc, pot, n, s));
     c->launches += ((q.terms & 1) ? 1 : 0) + ((q.terms & 2) ? 1 : 0) + 1;
     CK(cudaEventRecordWithFlags(c->ev[5], s, cudaEventRecordExternal));
     CK(cudaMemcpyAsync(c->ctr_h, c->ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s));
@@ -1271,7 +1272,7 @@ static void capture_graph(fmm_ctx* c, const fmm_ctx::GraphKey& key, const double
     // the work is recorded on the context's capture stream; replays launch on the caller's stream
     const int saved_launches = c->launches;
     cudaGraphExec_t head = capture_part(c, [&] { return enqueue_graph_head(c, pos, mass, active, n, q, box_off, nbox); });
-    cudaGraphExec_t rest = head ? capture_part(c, [&] { return enqueue_graph_rest(c, n, q, acc, pot, nbox); }) : nullptr;
+    cudaGraphExec_t rest = head ? capture_part(c, [&] { return enqueue_graph_rest(c, active, n, q, acc, pot, nbox); }) : nullptr;
     c->graph_launches = c->launches + c->t.n_launches;  // both parts
     c->launches = saved_launches;
     if (!head || !rest) {
@@ -1666,7 +1667,7 @@ extern "C" fmm_status fmm_compute_forces_dual(fmm_ctx* c, const double* pos, con
     if (st != FMM_OK) return st;
     CK(fmm_launch_compose_perm(t.idx, c->d_idx, na, c->d_perm, s));
     c->launches += 1;
-    return interact_and_finish(c, q, eps, acc, pot, n, na, c->d_perm);
+    return interact_and_finish(c, q, eps, nullptr, acc, pot, n, na, c->d_perm);
 }
 
 extern "C" fmm_status fmm_compute_forces_batch(fmm_ctx* c, const double* pos, const float* mass,

@@ -384,9 +384,11 @@ struct InteractArgs {
 cudaError_t fmm_launch_items(DevTree& t, DevWalk& w, DevCounters* ctr, int chunk, cudaStream_t s);
 cudaError_t fmm_launch_pp(DevTree& t, DevWalk& w, DevCounters* ctr, const InteractArgs& a, cudaStream_t s);
 cudaError_t fmm_launch_pc(DevTree& t, DevWalk& w, DevCounters* ctr, const InteractArgs& a, cudaStream_t s);
-// perm: sorted sink -> index in acc/pot (NULL: the tree's own order t.idx)
-cudaError_t fmm_launch_l2p_out(DevTree& t, DevWalk& w, DevCounters* ctr, const InteractArgs& a, float* acc,
-                               float* pot, long long n, cudaStream_t s, const unsigned int* perm = nullptr);
+// perm: sorted sink -> index in acc/pot (NULL: the tree's own order t.idx, the n particles of the call
+// with the flags active, or all of them, of which about n_active are sinks)
+cudaError_t fmm_launch_l2p_out(DevTree& t, DevWalk& w, DevCounters* ctr, const InteractArgs& a,
+                               const unsigned char* active, long long n_active, float* acc, float* pot, long long n,
+                               cudaStream_t s, const unsigned int* perm = nullptr);
 int fmm_interact_blocks(int device);
 
 // dual.cu

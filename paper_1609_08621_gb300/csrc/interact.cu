@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(ITHREADS) k_l2p_out(const Group* __restrict__ 
                                                       const int* __restrict__ act, const int* __restrict__ cnact,
                                                       const unsigned int* __restrict__ perm, long long n,
                                                       float* __restrict__ acc, float* __restrict__ pot, int terms,
-                                                      const DevCounters* __restrict__ ctr)
+                                                      float4* __restrict__ out, const DevCounters* __restrict__ ctr)
 {
     __shared__ float Ls[IW][FMM_NL];
     if (fmm_overflowed(ctr)) return;
@@ -580,6 +580,10 @@ __global__ void __launch_bounds__(ITHREADS) k_l2p_out(const Group* __restrict__ 
                 az += acc_widen(lz, az);
                 aw += acc_widen(lw, aw);
             }
+            if (out) {  // one record, spread over the caller's arrays by k_out_split
+                out[po] = make_float4(acc_round(ax), acc_round(ay), acc_round(az), acc_round(aw));
+                continue;
+            }
             acc[po] = acc_round(ax);
             acc[n + po] = acc_round(ay);
             acc[2 * n + po] = acc_round(az);
@@ -587,6 +591,24 @@ __global__ void __launch_bounds__(ITHREADS) k_l2p_out(const Group* __restrict__ 
         }
         __syncwarp();
     }
+}
+
+// The output records of the active particles, in the caller's order, into the caller's arrays.  With
+// several boxes the records start as all ones (marked), and those still so are of particles that no
+// sink held.
+__global__ void k_out_split(const float4* __restrict__ out, const unsigned char* __restrict__ active, bool marked,
+                            long long n, float* __restrict__ acc, float* __restrict__ pot,
+                            const DevCounters* __restrict__ ctr)
+{
+    if (fmm_overflowed(ctr)) return;
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n || (active && active[i] == 0)) return;
+    const float4 v = out[i];
+    if (marked && (__float_as_uint(v.x) & __float_as_uint(v.y) & __float_as_uint(v.z) & __float_as_uint(v.w)) == ~0u) return;
+    acc[i] = v.x;
+    acc[n + i] = v.y;
+    acc[2 * n + i] = v.z;
+    if (pot) pot[i] = v.w;
 }
 
 int fmm_interact_blocks(int device)
@@ -722,23 +744,37 @@ cudaError_t fmm_launch_pc(DevTree& t, DevWalk& w, DevCounters* ctr, const Intera
     return cudaGetLastError();
 }
 
-cudaError_t fmm_launch_l2p_out(DevTree& t, DevWalk& w, DevCounters* ctr, const InteractArgs& a, float* acc,
-                               float* pot, long long n, cudaStream_t s, const unsigned int* perm)
+// From FMM_OUT_RECORDS particles on (their results no longer fit L2), a solve of the caller's own
+// particles writes each result as one 16-byte record in the caller's order and splits the records in a
+// streaming pass: a scattered store costs a DRAM sector whatever its size, and the four arrays cost
+// four of them per particle.  384^3 box 9.1 to 4.7 ms, 64 boxes 3.5 to 2.1; the 128^3 box, within L2, is
+// slower (0.186 to 0.201), and so is a 256^3 substep with a tenth active (0.73 to 0.86), where the
+// streaming pass reads flags and records of every particle: so at least a quarter must be active.
+#define FMM_OUT_RECORDS (1LL << 22)
+cudaError_t fmm_launch_l2p_out(DevTree& t, DevWalk& w, DevCounters* ctr, const InteractArgs& a,
+                               const unsigned char* active, long long n_active, float* acc, float* pot, long long n,
+                               cudaStream_t s, const unsigned int* perm)
 {
     // the group expansions also carry the Ewald correction of a periodic box (terms & 8), so they
     // are evaluated when either part is asked for
     const int terms = (t.per_R > 0 && (a.terms & 8)) ? (a.terms | 4) : a.terms;
+    // the radix tree's block, 32 bytes per particle, is free once the cells are built
+    float4* const out = !perm && n >= FMM_OUT_RECORDS && 4 * n_active >= n ? reinterpret_cast<float4*>(t.radix) : nullptr;
     if (!perm) perm = t.idx;
     const long long ng = t.cap_grid ? w.cap_groups : w.n_groups;
-    if (a.accumulate == 1)
-        k_l2p_out<double><<<grid_for(ng), ITHREADS, 0, s>>>(
-            w.groups, &ctr->n_groups, w.cap_groups, w.cap_item_pp, w.cap_item_pc, t.cen, t.bucket_of, t.bucket_cell,
-            t.off, w.Lg, w.cnt_pp, w.base_pp, w.part_pp, w.cnt_pc, w.base_pc, w.part_pc, t.act, t.cnact, perm, n, acc, pot,
-            terms, ctr);
-    else
-        k_l2p_out<float><<<grid_for(ng), ITHREADS, 0, s>>>(
-            w.groups, &ctr->n_groups, w.cap_groups, w.cap_item_pp, w.cap_item_pc, t.cen, t.bucket_of, t.bucket_cell,
-            t.off, w.Lg, w.cnt_pp, w.base_pp, w.part_pp, w.cnt_pc, w.base_pc, w.part_pc, t.act, t.cnact, perm, n, acc, pot,
-            terms, ctr);
+    const bool marked = t.nbox > 1;
+    if (out && marked) {
+        const cudaError_t e = cudaMemsetAsync(out, 0xff, sizeof(float4) * (size_t)n, s);
+        if (e != cudaSuccess) return e;
+    }
+    auto kernel = a.accumulate == 1 ? k_l2p_out<double> : k_l2p_out<float>;
+    kernel<<<grid_for(ng), ITHREADS, 0, s>>>(w.groups, &ctr->n_groups, w.cap_groups, w.cap_item_pp, w.cap_item_pc, t.cen,
+                                             t.bucket_of, t.bucket_cell, t.off, w.Lg, w.cnt_pp, w.base_pp, w.part_pp,
+                                             w.cnt_pc, w.base_pc, w.part_pc, t.act, t.cnact, perm, n, acc, pot, terms,
+                                             out, ctr);
+    if (out) {
+        k_out_split<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(out, active, marked, n, acc, pot, ctr);
+        t.n_launches += 1;
+    }
     return cudaGetLastError();
 }
