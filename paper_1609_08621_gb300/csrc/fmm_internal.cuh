@@ -116,7 +116,6 @@ struct __align__(16) Group {
 };
 
 #define FMM_LIST_CHUNK 64  // default list entries per PP / PC work item
-#define FMM_LOCAL_RANGE 512  // local entries per warp range of the own-expansion kernel
 #define FMM_GMAX 64       // sink slots per group
 #define FMM_LOCAL_STEP 4  // walk levels between those whose cells' local expansions are evaluated
 #define FMM_MAX_LEVELS 192  // walk levels: tree depth + 1 (63 key bits + 31 position bits at most)

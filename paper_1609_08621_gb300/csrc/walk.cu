@@ -563,13 +563,20 @@ __global__ void __launch_bounds__(WALK_THREADS, MODE == 1 ? 4 : FMM_WALK_MINB) k
 #define LOCAL_THREADS (LOCAL_WPB * 32)
 
 // Own local expansions over the flat list of all local entries (every walked sink's CC and CP
-// entries, contiguous per sink).  A warp takes a range of about LF_ENTRIES entries, moved to the
-// next sink boundaries so that no sink is split between warps, and walks it in chunks of 32, one
-// entry per lane, so lanes stay busy whatever the list lengths.  Each sink's 56 coefficients are
+// entries, contiguous per sink).  A warp takes ranges of the list, moved to the next sink boundaries so
+// that no sink is split between warps, and walks each in chunks of 32, one entry per lane, so lanes
+// stay busy whatever the list lengths.  Each sink's 56 coefficients are
 // added strictly in list order (runs of equal sink along the lanes, a run that continues into
 // the next chunk carried on): the result depends only on the sink's own list, not on where the
 // list lies in the flat array or which warp took it.
-#define LF_ENTRIES FMM_LOCAL_RANGE
+//
+// A range is about a sixteenth of a warp's share of the list, so that the last turn's idle warps cost
+// little, but at least 64 entries (every range ends in a part-filled chunk; short lists then still
+// reach all SMs) and at most 8192.  Walk phase with ranges of 512 whatever the list, against this: 384^3
+// box 42.5 to 41.4 ms, 256^3 substep 14.0 to 13.5, 128^3 2.74 to 2.62, 4096 particles 0.31 to 0.265.
+#define LF_TURNS 16
+#define LF_MAX 8192
+#define LF_MIN 64
 
 // Centres enter as float pairs (cen_diff): the sink's (hk, lk), a cell's from cen, a particle's
 // from posf (hi, and its mass) and plo (lo); a source in a periodic copy has its pair shifted
@@ -660,12 +667,14 @@ __global__ void __launch_bounds__(LOCAL_THREADS, FMM_LOCAL_MINB) k_local_flat(
         total = min(start + (long long)__ldcg(lv + level), cap_cc);
     }
     if (start >= total) return;
-    const long long nranges = fmm_ceil_div(total - start, LF_ENTRIES);
+    // ranges of whole chunks, about LF_TURNS per warp
+    const long long len = min((long long)LF_MAX, max((long long)LF_MIN, (total - start) / (nw * LF_TURNS) / 32 * 32));
+    const long long nranges = fmm_ceil_div(total - start, len);
     const int c0 = lane, c1 = lane + 32;  // this lane's coefficients in the reduction
     int nent = 0;
     for (long long r = gw; r < nranges; r += nw) {
-        const long long r0 = local_boundary(start + r * LF_ENTRIES, total, cc_sink, lcc_off, lcc_len);
-        const long long r1 = local_boundary(start + (r + 1) * LF_ENTRIES, total, cc_sink, lcc_off, lcc_len);
+        const long long r0 = local_boundary(start + r * len, total, cc_sink, lcc_off, lcc_len);
+        const long long r1 = local_boundary(start + (r + 1) * len, total, cc_sink, lcc_off, lcc_len);
         float carry0 = 0.0f, carry1 = 0.0f;
         int carry_sink = -1;
         // entries and sinks are read a chunk ahead: of a chunk's two dependent rounds of loads (they, then
@@ -1074,24 +1083,40 @@ cudaError_t fmm_launch_local_level(DevTree& t, DevWalk& w, DevCounters* ctr, flo
     return cudaGetLastError();
 }
 
+// resident blocks per SM of the local-expansion kernels, looked up once per device
+template <int KIND>
+static int local_resident(int dev)
+{
+    static std::atomic<int> table[64];
+    const bool cached = dev >= 0 && dev < 64;
+    int b = cached ? table[dev].load(std::memory_order_relaxed) : 0;
+    if (b > 0) return b;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_local_flat<KIND>, LOCAL_THREADS, 0) != cudaSuccess || b < 1) b = 1;
+    if (cached) table[dev].store(b, std::memory_order_relaxed);
+    return b;
+}
+
 // Grid sizes for a level with about n_cc / n_cp local entries and n_cells walked cells (counts of
-// the context's previous walk; negative: unknown, the full persistent grids).  Never below two
+// the context's previous walk; negative: unknown, the full persistent grids).  A full grid is what the
+// SMs hold at once: its warps take ranges with a fixed stride, so blocks beyond that are a second wave
+// (12 blocks per SM with 8 resident left a quarter of the M2L pass's warps idle).  Never below two
 // blocks per SM: counts that changed since cost a level at most a few-fold, not its parallelism.
 LocalGrids fmm_local_grids(const DevWalk& w, long long n_cc, long long n_cp, long long n_cells)
 {
+    (void)w;
     int sms = 152, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const long long full = w.n_warps / LOCAL_WPB, full_down = (long long)sms * 8, floor = 2LL * sms;
-    auto flat = [&](long long e) {
+    const long long full_down = (long long)sms * 8, floor = 2LL * sms;
+    auto flat = [&](long long e, long long full) {
         if (e < 0) return (unsigned)full;
-        // a quarter more warps than ranges
-        const long long warps = fmm_ceil_div(e, LF_ENTRIES) * 5 / 4 + 1;
+        // a quarter more warps than the shortest ranges
+        const long long warps = fmm_ceil_div(e, LF_MIN) * 5 / 4 + 1;
         return (unsigned)std::max(std::min(floor, full), std::min(full, fmm_ceil_div(warps, LOCAL_WPB)));
     };
     LocalGrids g;
-    g.cc = flat(n_cc);
-    g.cp = flat(n_cp);
+    g.cc = flat(n_cc, (long long)sms * local_resident<0>(dev));
+    g.cp = flat(n_cp, (long long)sms * local_resident<1>(dev));
     g.down = n_cells < 0 ? (unsigned)full_down
                          : (unsigned)std::max(std::min(floor, full_down),
                                               std::min(full_down, fmm_ceil_div(n_cells * 5 / 4 + 1, LD_THREADS / 32)));
