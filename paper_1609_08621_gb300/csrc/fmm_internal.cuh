@@ -33,7 +33,7 @@ __host__ __device__ __forceinline__ Com4 make_com4(double x, double y, double z,
 // One tree cell as the walk reads it: 64 bytes, four aligned 16-byte loads.
 //   a = (centre of mass, single precision, and R_O = b_max / theta)
 //   b = (bounding box lo, single precision, and b_max)
-//   c = (bounding box hi, single precision, and unused)
+//   c = (bounding box hi, single precision, and log2 of the count, a feature of the learned criterion)
 //   d = (child0, child1, first, count); child0 = -1 for a bucket
 struct __align__(16) WalkNode {
     float4 a, b, c;
@@ -216,7 +216,7 @@ struct DevTree {
     double *bmax = nullptr;
     float *rec = nullptr;        // FMM_NREC per cell
     WalkNode *node = nullptr;
-    float4 *mnorm = nullptr;     // per cell: |M2|/(M b^2), |M4|/(M b^4), M (float), 0
+    float4 *mnorm = nullptr;     // per cell: |M2|/(M b^2), |M4|/(M b^4), M (float), log10 M
     float *amin = nullptr;       // per cell: smallest |a| estimate of its particles (learned criterion)
     float *L = nullptr;          // FMM_NL per cell: own local expansion of walked cells
     // several independent boxes: box b holds sorted particles [box_off[b], box_off[b+1])

@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(128) k_audit_labels(
         for (int o = 16; o > 0; o >>= 1) err = fmaxf(err, __shfl_xor_sync(FMM_FULL_MASK, err, o));
         if (lane == 0) {
             labels[q] = log10f(err + 1e-12f);
-            mlp_pair_features(node[k], node[s], mnorm[s], amin[k], eps, feats + q * MLP_F);
+            mlp_pair_features(node[k], node[s], mnorm[s], mlp_log_accel(amin[k]), eps, feats + q * MLP_F);
         }
     }
 }

@@ -181,8 +181,10 @@ __device__ __forceinline__ int mlp_band(const WalkNode& K, const WalkNode& S, fl
 // the 8 features of a (sink k, source s) pair: b_max(s)/d, b_max(k)/d, eps/d,
 // log10(M_s / (d^2 a_k)) (the source's monopole field at the sink relative to the sink's smallest
 // particle acceleration a_k), log2 N_s, log2 N_k, |M2|_F/(M b^2), |M4|_F/(M b^4) of the source.
-// mn = (|M2| norm, |M4| norm, M_s, -) of the source; ak = a_k (clamped below at 1e-30).
-__device__ __forceinline__ void mlp_pair_features(const WalkNode& K, const WalkNode& S, float4 mn, float ak, float eps,
+// mn = (|M2| norm, |M4| norm, M_s, log10 M_s) of the source; la = mlp_log_accel(a_k).  The logarithms of one
+// cell alone are taken once per cell (mn.w, and log2 N in the nodes' c.w) and per sink (la).
+__device__ __forceinline__ float mlp_log_accel(float ak) { return log10f(fmaxf(ak, 1e-30f)); }
+__device__ __forceinline__ void mlp_pair_features(const WalkNode& K, const WalkNode& S, float4 mn, float la, float eps,
                                                   float* f)
 {
     const float dx = K.a.x - S.a.x, dy = K.a.y - S.a.y, dz = K.a.z - S.a.z;
@@ -192,9 +194,9 @@ __device__ __forceinline__ void mlp_pair_features(const WalkNode& K, const WalkN
     f[0] = S.b.w * id;
     f[1] = K.b.w * id;
     f[2] = eps * id;
-    f[3] = log10f(mn.z) - log10f(d2) - log10f(fmaxf(ak, 1e-30f));
-    f[4] = log2f((float)S.d.w);
-    f[5] = log2f((float)K.d.w);
+    f[3] = mn.w - log10f(d2) - la;
+    f[4] = S.c.w;
+    f[5] = K.c.w;
     f[6] = mn.x;
     f[7] = mn.y;
 }

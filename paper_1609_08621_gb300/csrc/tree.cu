@@ -795,13 +795,14 @@ __global__ void k_nodes(const unsigned int* __restrict__ ncell, float theta, con
     cen[2 * c] = make_float4(hx, hy, hz, 0.0f);
     cen[2 * c + 1] = make_float4(lx, ly, lz, 0.0f);
     w.b = make_float4(fmm_d2f_rn(clo[3 * c]), fmm_d2f_rn(clo[3 * c + 1]), fmm_d2f_rn(clo[3 * c + 2]), bm);
-    w.c = make_float4(fmm_d2f_rn(chi[3 * c]), fmm_d2f_rn(chi[3 * c + 1]), fmm_d2f_rn(chi[3 * c + 2]), 0.0f);
+    w.c = make_float4(fmm_d2f_rn(chi[3 * c]), fmm_d2f_rn(chi[3 * c + 1]), fmm_d2f_rn(chi[3 * c + 2]),
+                      log2f((float)cnt));
     w.d = make_int4(cchild[2 * c], cchild[2 * c + 1], cfirst[c], cnt);
     node[c] = w;
     // multipole norms for the learned criterion: |M2|_F / (M b^2), |M4|_F / (M b^4), both in [0, 1];
     // cells smaller than 1e-7 of the box (coincident particles) report 0
     const float mass32 = fmm_d2f_rn(cm.w);
-    float4 mn = make_float4(0.0f, 0.0f, mass32, 0.0f);
+    float4 mn = make_float4(0.0f, 0.0f, mass32, log10f(mass32));
     if (bm > 1e-7f && cnt > 1) {
         const float b2 = bm * bm, s2 = 1.0f / (mass32 * b2), s4 = s2 / b2;
         float n2, n4;

@@ -233,7 +233,7 @@ __device__ __forceinline__ void walk_sinks(const WalkIO& w, const unsigned long 
         // fixed tree's groups around it
         const bool kg = K.d.w <= w.group && !(w.nogroup && w.nogroup[k]);
         const float rk = K.a.w, bk = K.b.w, rk15 = __fmul_rn(1.5f, rk);
-        const float ak = MODE == 1 ? w.amin[k] : 0.0f;
+        const float ak = MODE == 1 ? w.amin[k] : 0.0f, la = MODE == 1 ? mlp_log_accel(ak) : 0.0f;
         const unsigned int* const cl = w.cl_cur + w.f_cloff[fi];
         const int ncl = w.f_cllen[fi];
         unsigned int* const X = kg ? C : D;  // a group's PC entries, any other sink's deferred ones
@@ -277,7 +277,7 @@ __device__ __forceinline__ void walk_sinks(const WalkIO& w, const unsigned long 
                                 band = acc ? 1 : 2;  // no acceleration estimate: the fixed criterion decides
                             } else if (band == 3) {
                                 float f[MLP_F];
-                                mlp_pair_features(K, S, w.mnorm[entry_index(e, ib)], ak, w.eps, f);
+                                mlp_pair_features(K, S, w.mnorm[entry_index(e, ib)], la, w.eps, f);
                                 band = mlp_surrogate(reinterpret_cast<const float*>(walk_smem + MLPP_SUR), f, te, w.tau,
                                                      w.margin);
                             }
@@ -419,7 +419,7 @@ __device__ __forceinline__ void walk_sinks(const WalkIO& w, const unsigned long 
                 if (lane < cnt) {
                     pe = W[b + lane];
                     const unsigned int j = entry_index(pe, ib);
-                    mlp_pair_features(K, w.node[j], w.mnorm[j], ak, w.eps, f);
+                    mlp_pair_features(K, w.node[j], w.mnorm[j], la, w.eps, f);
                 }
                 const float pred = mlp_predict_warp(walk_smem, mlp_scratch, f, lane,
                                                     cnt == 32 ? FMM_FULL_MASK : (1u << cnt) - 1u);
