@@ -82,42 +82,86 @@ __device__ __forceinline__ double pow2_scale(double dt0, int k)
 // FP64 issues at 1/64 of the FP32 rate on this GPU: the kicks and the drift are FP64 arithmetic, while
 // the widening of the FP32 accelerations and the box check of the new position use the encodings
 // (f64bits.cuh) and give the same values.
-__global__ void k_kick_drift(double* __restrict__ pos, double* __restrict__ vel, const float* __restrict__ acc,
-                             unsigned char* __restrict__ rung, unsigned char* __restrict__ active_next, long long n,
-                             double eps, double dt0, int R, float t0, long long s, int closing,
-                             unsigned int* __restrict__ status)
+//
+// A warp pays for an FP64 instruction in full however few of its lanes are active, and on a substep
+// nearly every warp holds some of the active tenth.  So a block gathers its active particles in shared
+// memory and kicks them with as few warps as hold them; the drift, of every particle, follows.  256^3 box,
+// a tenth active: 0.365 ms, 4.1 TB/s, against 0.465 with every particle kicked in its own lane (6 blocks per
+// SM; 0.39 with 5, 0.41 with 4).
+#define KD_THREADS 256
+__global__ void __launch_bounds__(KD_THREADS, 6) k_kick_drift(
+    double* __restrict__ pos, double* __restrict__ vel, const float* __restrict__ acc, unsigned char* __restrict__ rung,
+    unsigned char* __restrict__ active_next, long long n, double eps, double dt0, int R, float t0, long long s, int closing,
+    unsigned int* __restrict__ status)
 {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int r = rung[i];
-    double vx = vel[i], vy = vel[n + i], vz = vel[2 * n + i];
-    if ((s & ((1LL << (R - r)) - 1)) == 0) {
-        float fx = acc[i], fy = acc[n + i], fz = acc[2 * n + i];
-        double ax = fmm_f2d(fx), ay = fmm_f2d(fy), az = fmm_f2d(fz);
-        if (closing) {
-            double hk = pow2_scale(dt0, r + 1);
-            vx += ax * hk;
-            vy += ay * hk;
-            vz += az * hk;
-        }
-        int rt = target_rung(fx, fy, fz, eps, dt0, R, t0);
-        int rn = rt;
-        if (rt < r) {
-            rn = rt;
-            while (rn < r && (s & ((1LL << (R - rn)) - 1)) != 0) rn++;
-        }
-        r = rn;
-        rung[i] = (unsigned char)r;
-        double hk = pow2_scale(dt0, r + 1);
-        vx += ax * hk;
-        vy += ay * hk;
-        vz += az * hk;
-        vel[i] = vx;
-        vel[n + i] = vy;
-        vel[2 * n + i] = vz;
+    __shared__ double v[3][KD_THREADS];
+    __shared__ unsigned char rs[KD_THREADS], list[KD_THREADS];
+    __shared__ int count;
+    const int tid = threadIdx.x;
+    const long long first = (long long)blockIdx.x * KD_THREADS, i = first + tid;
+    const bool valid = i < n;
+    if (tid == 0) count = 0;
+    int r = 0;
+    double vx = 0.0, vy = 0.0, vz = 0.0, x = 0.0, y = 0.0, z = 0.0;
+    if (valid) {
+        r = rung[i];
+        vx = vel[i];
+        vy = vel[n + i];
+        vz = vel[2 * n + i];
+        x = pos[i];
+        y = pos[n + i];
+        z = pos[2 * n + i];
     }
-    double h = pow2_scale(dt0, R);
-    double x = pos[i] + vx * h, y = pos[n + i] + vy * h, z = pos[2 * n + i] + vz * h;
+    const bool active = valid && (s & ((1LL << (R - r)) - 1)) == 0;
+    __syncthreads();
+    const unsigned int m = __ballot_sync(FMM_FULL_MASK, active);
+    int at = 0;
+    if ((tid & 31) == 0 && m) at = atomicAdd(&count, __popc(m));
+    at = __shfl_sync(FMM_FULL_MASK, at, 0) + __popc(m & fmm_lanemask_lt());
+    if (active) {
+        list[at] = (unsigned char)tid;
+        rs[tid] = (unsigned char)r;
+        v[0][tid] = vx;
+        v[1][tid] = vy;
+        v[2][tid] = vz;
+    }
+    __syncthreads();
+    if (tid < count) {
+        const int q = list[tid], ro = rs[q];
+        const long long j = first + q;
+        double wx = v[0][q], wy = v[1][q], wz = v[2][q];
+        const float fx = acc[j], fy = acc[n + j], fz = acc[2 * n + j];
+        const double ax = fmm_f2d(fx), ay = fmm_f2d(fy), az = fmm_f2d(fz);
+        if (closing) {
+            const double hk = pow2_scale(dt0, ro + 1);
+            wx += ax * hk;
+            wy += ay * hk;
+            wz += az * hk;
+        }
+        int rn = target_rung(fx, fy, fz, eps, dt0, R, t0);
+        while (rn < ro && (s & ((1LL << (R - rn)) - 1)) != 0) rn++;
+        const double hk = pow2_scale(dt0, rn + 1);
+        wx += ax * hk;
+        wy += ay * hk;
+        wz += az * hk;
+        v[0][q] = wx;
+        v[1][q] = wy;
+        v[2][q] = wz;
+        rs[q] = (unsigned char)rn;
+    }
+    __syncthreads();
+    if (!valid) return;
+    if (active) {
+        r = rs[tid];
+        rung[i] = (unsigned char)r;
+        vel[i] = vx = v[0][tid];
+        vel[n + i] = vy = v[1][tid];
+        vel[2 * n + i] = vz = v[2][tid];
+    }
+    const double h = pow2_scale(dt0, R);
+    x += vx * h;
+    y += vy * h;
+    z += vz * h;
     if (!(fmm_in_unit(x) && fmm_in_unit(y) && fmm_in_unit(z))) atomicOr(status, FMM_DEV_ERR_ARG);
     pos[i] = x;
     pos[n + i] = y;
@@ -130,7 +174,7 @@ cudaError_t fmm_launch_kick_drift(double* pos, double* vel, const float* acc, un
                                   unsigned char* active_next, long long n, double eps, double dt0, int max_rung,
                                   int substep, int closing, DevCounters* ctr, cudaStream_t s)
 {
-    k_kick_drift<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(pos, vel, acc, rung, active_next, n, eps, dt0,
+    k_kick_drift<<<(unsigned)fmm_ceil_div(n, KD_THREADS), KD_THREADS, 0, s>>>(pos, vel, acc, rung, active_next, n, eps, dt0,
                                                                 max_rung, rung_threshold(eps, dt0), substep, closing, &ctr->status);
     return cudaGetLastError();
 }
