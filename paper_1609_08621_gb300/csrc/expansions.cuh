@@ -216,76 +216,145 @@ __device__ __forceinline__ void fmm_p2m_acc(float m, float yx, float yy, float y
     M[31] += m * y004;
 }
 
+#ifdef __CUDA_ARCH__
+#define FMM_MUL(a, b) __fmul_rn(a, b)
+#else
+#define FMM_MUL(a, b) ((a) * (b))
+#endif
 /* child moments about its own centre -> parent centre, t = com_child - com_parent */
 __device__ __forceinline__ void fmm_m2m_acc(const float* __restrict__ Mc, float tx, float ty, float tz,
                                             float* __restrict__ Mp)
 {
-    const float t100 = tx;
-    const float t010 = ty;
-    const float t001 = tz;
-    const float t200 = t100 * tx;
-    const float t110 = t010 * tx;
-    const float t101 = t001 * tx;
-    const float t020 = t010 * ty;
-    const float t011 = t001 * ty;
-    const float t002 = t001 * tz;
-    const float t300 = t200 * tx;
-    const float t210 = t110 * tx;
-    const float t201 = t101 * tx;
-    const float t120 = t020 * tx;
-    const float t111 = t011 * tx;
-    const float t102 = t002 * tx;
-    const float t030 = t020 * ty;
-    const float t021 = t011 * ty;
-    const float t012 = t002 * ty;
-    const float t003 = t002 * tz;
-    const float t400 = t300 * tx;
-    const float t310 = t210 * tx;
-    const float t301 = t201 * tx;
-    const float t220 = t120 * tx;
-    const float t211 = t111 * tx;
-    const float t202 = t102 * tx;
-    const float t130 = t030 * tx;
-    const float t121 = t021 * tx;
-    const float t112 = t012 * tx;
-    const float t103 = t003 * tx;
-    const float t040 = t030 * ty;
-    const float t031 = t021 * ty;
-    const float t022 = t012 * ty;
-    const float t013 = t003 * ty;
-    const float t004 = t003 * tz;
-    Mp[0] += Mc[0];
-    Mp[1] += t200 * Mc[0] + Mc[1];
-    Mp[2] += t110 * Mc[0] + Mc[2];
-    Mp[3] += t101 * Mc[0] + Mc[3];
-    Mp[4] += t020 * Mc[0] + Mc[4];
-    Mp[5] += t011 * Mc[0] + Mc[5];
-    Mp[6] += t002 * Mc[0] + Mc[6];
-    Mp[7] += t300 * Mc[0] + 3.0f * tx * Mc[1] + Mc[7];
-    Mp[8] += t210 * Mc[0] + ty * Mc[1] + 2.0f * tx * Mc[2] + Mc[8];
-    Mp[9] += t201 * Mc[0] + tz * Mc[1] + 2.0f * tx * Mc[3] + Mc[9];
-    Mp[10] += t120 * Mc[0] + 2.0f * ty * Mc[2] + tx * Mc[4] + Mc[10];
-    Mp[11] += t111 * Mc[0] + tz * Mc[2] + ty * Mc[3] + tx * Mc[5] + Mc[11];
-    Mp[12] += t102 * Mc[0] + 2.0f * tz * Mc[3] + tx * Mc[6] + Mc[12];
-    Mp[13] += t030 * Mc[0] + 3.0f * ty * Mc[4] + Mc[13];
-    Mp[14] += t021 * Mc[0] + tz * Mc[4] + 2.0f * ty * Mc[5] + Mc[14];
-    Mp[15] += t012 * Mc[0] + 2.0f * tz * Mc[5] + ty * Mc[6] + Mc[15];
-    Mp[16] += t003 * Mc[0] + 3.0f * tz * Mc[6] + Mc[16];
-    Mp[17] += t400 * Mc[0] + 6.0f * t200 * Mc[1] + 4.0f * tx * Mc[7] + Mc[17];
-    Mp[18] += t310 * Mc[0] + 3.0f * t110 * Mc[1] + 3.0f * t200 * Mc[2] + ty * Mc[7] + 3.0f * tx * Mc[8] + Mc[18];
-    Mp[19] += t301 * Mc[0] + 3.0f * t101 * Mc[1] + 3.0f * t200 * Mc[3] + tz * Mc[7] + 3.0f * tx * Mc[9] + Mc[19];
-    Mp[20] += t220 * Mc[0] + t020 * Mc[1] + 4.0f * t110 * Mc[2] + t200 * Mc[4] + 2.0f * ty * Mc[8] + 2.0f * tx * Mc[10] + Mc[20];
-    Mp[21] += t211 * Mc[0] + t011 * Mc[1] + 2.0f * t101 * Mc[2] + 2.0f * t110 * Mc[3] + t200 * Mc[5] + tz * Mc[8] + ty * Mc[9] + 2.0f * tx * Mc[11] + Mc[21];
-    Mp[22] += t202 * Mc[0] + t002 * Mc[1] + 4.0f * t101 * Mc[3] + t200 * Mc[6] + 2.0f * tz * Mc[9] + 2.0f * tx * Mc[12] + Mc[22];
-    Mp[23] += t130 * Mc[0] + 3.0f * t020 * Mc[2] + 3.0f * t110 * Mc[4] + 3.0f * ty * Mc[10] + tx * Mc[13] + Mc[23];
-    Mp[24] += t121 * Mc[0] + 2.0f * t011 * Mc[2] + t020 * Mc[3] + t101 * Mc[4] + 2.0f * t110 * Mc[5] + tz * Mc[10] + 2.0f * ty * Mc[11] + tx * Mc[14] + Mc[24];
-    Mp[25] += t112 * Mc[0] + t002 * Mc[2] + 2.0f * t011 * Mc[3] + 2.0f * t101 * Mc[5] + t110 * Mc[6] + 2.0f * tz * Mc[11] + ty * Mc[12] + tx * Mc[15] + Mc[25];
-    Mp[26] += t103 * Mc[0] + 3.0f * t002 * Mc[3] + 3.0f * t101 * Mc[6] + 3.0f * tz * Mc[12] + tx * Mc[16] + Mc[26];
-    Mp[27] += t040 * Mc[0] + 6.0f * t020 * Mc[4] + 4.0f * ty * Mc[13] + Mc[27];
-    Mp[28] += t031 * Mc[0] + 3.0f * t011 * Mc[4] + 3.0f * t020 * Mc[5] + tz * Mc[13] + 3.0f * ty * Mc[14] + Mc[28];
-    Mp[29] += t022 * Mc[0] + t002 * Mc[4] + 4.0f * t011 * Mc[5] + t020 * Mc[6] + 2.0f * tz * Mc[14] + 2.0f * ty * Mc[15] + Mc[29];
-    Mp[30] += t013 * Mc[0] + 3.0f * t002 * Mc[5] + 3.0f * t011 * Mc[6] + 3.0f * tz * Mc[15] + ty * Mc[16] + Mc[30];
-    Mp[31] += t004 * Mc[0] + 6.0f * t002 * Mc[6] + 4.0f * tz * Mc[16] + Mc[31];
+    float s0 = Mc[0];
+    float s1 = 0.0f;
+    float s2 = 0.0f;
+    float s3 = 0.0f;
+    float s4 = Mc[1];
+    float s5 = Mc[2];
+    float s6 = Mc[3];
+    float s7 = Mc[4];
+    float s8 = Mc[5];
+    float s9 = Mc[6];
+    float s10 = Mc[7];
+    float s11 = Mc[8];
+    float s12 = Mc[9];
+    float s13 = Mc[10];
+    float s14 = Mc[11];
+    float s15 = Mc[12];
+    float s16 = Mc[13];
+    float s17 = Mc[14];
+    float s18 = Mc[15];
+    float s19 = Mc[16];
+    float s20 = Mc[17];
+    float s21 = Mc[18];
+    float s22 = Mc[19];
+    float s23 = Mc[20];
+    float s24 = Mc[21];
+    float s25 = Mc[22];
+    float s26 = Mc[23];
+    float s27 = Mc[24];
+    float s28 = Mc[25];
+    float s29 = Mc[26];
+    float s30 = Mc[27];
+    float s31 = Mc[28];
+    float s32 = Mc[29];
+    float s33 = Mc[30];
+    float s34 = Mc[31];
+    const float x2 = FMM_MUL(tx, tx), x3 = FMM_MUL(x2, tx), x4 = FMM_MUL(x3, tx);
+    s20 = fmaf(x4, s0, fmaf(FMM_MUL(4.0f, x3), s1, fmaf(FMM_MUL(6.0f, x2), s4, fmaf(FMM_MUL(4.0f, tx), s10, s20))));
+    s10 = fmaf(x3, s0, fmaf(FMM_MUL(3.0f, x2), s1, fmaf(FMM_MUL(3.0f, tx), s4, s10)));
+    s21 = fmaf(x3, s2, fmaf(FMM_MUL(3.0f, x2), s5, fmaf(FMM_MUL(3.0f, tx), s11, s21)));
+    s22 = fmaf(x3, s3, fmaf(FMM_MUL(3.0f, x2), s6, fmaf(FMM_MUL(3.0f, tx), s12, s22)));
+    s4 = fmaf(x2, s0, fmaf(FMM_MUL(2.0f, tx), s1, s4));
+    s11 = fmaf(x2, s2, fmaf(FMM_MUL(2.0f, tx), s5, s11));
+    s12 = fmaf(x2, s3, fmaf(FMM_MUL(2.0f, tx), s6, s12));
+    s23 = fmaf(x2, s7, fmaf(FMM_MUL(2.0f, tx), s13, s23));
+    s24 = fmaf(x2, s8, fmaf(FMM_MUL(2.0f, tx), s14, s24));
+    s25 = fmaf(x2, s9, fmaf(FMM_MUL(2.0f, tx), s15, s25));
+    s1 = fmaf(tx, s0, s1);
+    s5 = fmaf(tx, s2, s5);
+    s6 = fmaf(tx, s3, s6);
+    s13 = fmaf(tx, s7, s13);
+    s14 = fmaf(tx, s8, s14);
+    s15 = fmaf(tx, s9, s15);
+    s26 = fmaf(tx, s16, s26);
+    s27 = fmaf(tx, s17, s27);
+    s28 = fmaf(tx, s18, s28);
+    s29 = fmaf(tx, s19, s29);
+    const float y2 = FMM_MUL(ty, ty), y3 = FMM_MUL(y2, ty), y4 = FMM_MUL(y3, ty);
+    s30 = fmaf(y4, s0, fmaf(FMM_MUL(4.0f, y3), s2, fmaf(FMM_MUL(6.0f, y2), s7, fmaf(FMM_MUL(4.0f, ty), s16, s30))));
+    s16 = fmaf(y3, s0, fmaf(FMM_MUL(3.0f, y2), s2, fmaf(FMM_MUL(3.0f, ty), s7, s16)));
+    s26 = fmaf(y3, s1, fmaf(FMM_MUL(3.0f, y2), s5, fmaf(FMM_MUL(3.0f, ty), s13, s26)));
+    s31 = fmaf(y3, s3, fmaf(FMM_MUL(3.0f, y2), s8, fmaf(FMM_MUL(3.0f, ty), s17, s31)));
+    s7 = fmaf(y2, s0, fmaf(FMM_MUL(2.0f, ty), s2, s7));
+    s13 = fmaf(y2, s1, fmaf(FMM_MUL(2.0f, ty), s5, s13));
+    s17 = fmaf(y2, s3, fmaf(FMM_MUL(2.0f, ty), s8, s17));
+    s23 = fmaf(y2, s4, fmaf(FMM_MUL(2.0f, ty), s11, s23));
+    s27 = fmaf(y2, s6, fmaf(FMM_MUL(2.0f, ty), s14, s27));
+    s32 = fmaf(y2, s9, fmaf(FMM_MUL(2.0f, ty), s18, s32));
+    s2 = fmaf(ty, s0, s2);
+    s5 = fmaf(ty, s1, s5);
+    s8 = fmaf(ty, s3, s8);
+    s11 = fmaf(ty, s4, s11);
+    s14 = fmaf(ty, s6, s14);
+    s18 = fmaf(ty, s9, s18);
+    s21 = fmaf(ty, s10, s21);
+    s24 = fmaf(ty, s12, s24);
+    s28 = fmaf(ty, s15, s28);
+    s33 = fmaf(ty, s19, s33);
+    const float z2 = FMM_MUL(tz, tz), z3 = FMM_MUL(z2, tz), z4 = FMM_MUL(z3, tz);
+    s34 = fmaf(z4, s0, fmaf(FMM_MUL(4.0f, z3), s3, fmaf(FMM_MUL(6.0f, z2), s9, fmaf(FMM_MUL(4.0f, tz), s19, s34))));
+    s19 = fmaf(z3, s0, fmaf(FMM_MUL(3.0f, z2), s3, fmaf(FMM_MUL(3.0f, tz), s9, s19)));
+    s29 = fmaf(z3, s1, fmaf(FMM_MUL(3.0f, z2), s6, fmaf(FMM_MUL(3.0f, tz), s15, s29)));
+    s33 = fmaf(z3, s2, fmaf(FMM_MUL(3.0f, z2), s8, fmaf(FMM_MUL(3.0f, tz), s18, s33)));
+    s9 = fmaf(z2, s0, fmaf(FMM_MUL(2.0f, tz), s3, s9));
+    s15 = fmaf(z2, s1, fmaf(FMM_MUL(2.0f, tz), s6, s15));
+    s18 = fmaf(z2, s2, fmaf(FMM_MUL(2.0f, tz), s8, s18));
+    s25 = fmaf(z2, s4, fmaf(FMM_MUL(2.0f, tz), s12, s25));
+    s28 = fmaf(z2, s5, fmaf(FMM_MUL(2.0f, tz), s14, s28));
+    s32 = fmaf(z2, s7, fmaf(FMM_MUL(2.0f, tz), s17, s32));
+    s3 = fmaf(tz, s0, s3);
+    s6 = fmaf(tz, s1, s6);
+    s8 = fmaf(tz, s2, s8);
+    s12 = fmaf(tz, s4, s12);
+    s14 = fmaf(tz, s5, s14);
+    s17 = fmaf(tz, s7, s17);
+    s22 = fmaf(tz, s10, s22);
+    s24 = fmaf(tz, s11, s24);
+    s27 = fmaf(tz, s13, s27);
+    s31 = fmaf(tz, s16, s31);
+    Mp[0] += s0;
+    Mp[1] += s4;
+    Mp[2] += s5;
+    Mp[3] += s6;
+    Mp[4] += s7;
+    Mp[5] += s8;
+    Mp[6] += s9;
+    Mp[7] += s10;
+    Mp[8] += s11;
+    Mp[9] += s12;
+    Mp[10] += s13;
+    Mp[11] += s14;
+    Mp[12] += s15;
+    Mp[13] += s16;
+    Mp[14] += s17;
+    Mp[15] += s18;
+    Mp[16] += s19;
+    Mp[17] += s20;
+    Mp[18] += s21;
+    Mp[19] += s22;
+    Mp[20] += s23;
+    Mp[21] += s24;
+    Mp[22] += s25;
+    Mp[23] += s26;
+    Mp[24] += s27;
+    Mp[25] += s28;
+    Mp[26] += s29;
+    Mp[27] += s30;
+    Mp[28] += s31;
+    Mp[29] += s32;
+    Mp[30] += s33;
+    Mp[31] += s34;
 }
 
 /* traces of the moment tensors for the particle-cell kernel */
@@ -819,5 +888,5 @@ __device__ __forceinline__ void fmm_pc_acc2(const float* __restrict__ R, float2 
     fmm_pc_body2(S, rx, ry, rz, eps2, ax, ay, az, phip);
 }
 
-/* FP32 flops of the generated bodies (fmaf = 2): green 300, p2m 94, m2m 344, traces 22, norms 76, m2l 810, p2l 119, l2l 1095, l2p 499, pc 293, pc2 246 */
+/* FP32 flops of the generated bodies (fmaf = 2): green 300, p2m 94, m2m 242, traces 22, norms 76, m2l 810, p2l 119, l2l 1095, l2p 499, pc 293, pc2 246 */
 #define FMM_FLOPS_PC 246

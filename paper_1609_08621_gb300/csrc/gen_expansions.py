@@ -167,25 +167,39 @@ def gen_p2m():
 
 
 def gen_m2m():
-    """Shift child moments (about the child's centre) to the parent centre: y_p = y_c + t.
-    M_n(p) += sum_{k<=n} C(n,k) t^(n-k) M_k(c); the child's dipole is zero."""
-    L = ["/* child moments about its own centre -> parent centre, t = com_child - com_parent */",
+    """Shift child moments (about the child's centre) to the parent centre: y_p = y_c + t, one axis after
+    the other: M_n += sum_{i>=1} C(n_a, i) t_a^i M_(n - i e_a), an exact binomial shift along the axis, 35
+    multiply-adds per axis over the 35 moments to order 4.  The child's dipole is zero about its own
+    centre but not on the way, so the orders in between are all there; the parent's shifted dipoles
+    cancel and are dropped.  Every operation is written out (no contraction is left to the compiler), so
+    that the same shift spread over a warp's lanes gives the same bits."""
+    mi = [n for n in MI if sum(n) <= ORDER_M]
+    idx = {n: i for i, n in enumerate(mi)}
+    assert len(mi) == 35 and all(MSLOT[n] == (0 if i == 0 else i - 3) for i, n in enumerate(mi) if sum(n) != 1)
+    L = ["#ifdef __CUDA_ARCH__",
+         "#define FMM_MUL(a, b) __fmul_rn(a, b)",
+         "#else",
+         "#define FMM_MUL(a, b) ((a) * (b))",
+         "#endif",
+         "/* child moments about its own centre -> parent centre, t = com_child - com_parent */",
          "__device__ __forceinline__ void fmm_m2m_acc(const float* __restrict__ Mc, float tx, float ty, float tz,",
          "                                            float* __restrict__ Mp)", "{"]
-    L += emit_monomials("t", ORDER_M)
+    for n in mi:
+        L.append(f"    float s{idx[n]} = " + ("0.0f" if sum(n) == 1 else f"Mc[{MSLOT[n]}]") + ";")
+    for a, c in enumerate("xyz"):
+        L.append(f"    const float {c}2 = FMM_MUL(t{c}, t{c}), {c}3 = FMM_MUL({c}2, t{c}), {c}4 = FMM_MUL({c}3, t{c});")
+        pw = [None, f"t{c}", f"{c}2", f"{c}3", f"{c}4"]
+        for n in sorted(mi, key=lambda n: -n[a]):  # the highest power first: the lower ones are still unshifted
+            e = f"s{idx[n]}"
+            for i in range(1, n[a] + 1):
+                lo = tuple(v - (i if q == a else 0) for q, v in enumerate(n))
+                k = math.comb(n[a], i)
+                f = pw[i] if k == 1 else f"FMM_MUL({lit(k)}, {pw[i]})"
+                e = f"fmaf({f}, s{idx[lo]}, {e})"
+            if n[a]:
+                L.append(f"    s{idx[n]} = {e};")
     for n in MOM:
-        terms = []
-        for k in MOM:
-            if all(k[q] <= n[q] for q in range(3)):
-                binom = math.comb(n[0], k[0]) * math.comb(n[1], k[1]) * math.comb(n[2], k[2])
-                r = mono_ref("t", sub(n, k))
-                t = f"Mc[{MSLOT[k]}]"
-                if r is not None:
-                    t = f"{r} * {t}"
-                if binom != 1:
-                    t = f"{lit(binom)} * {t}"
-                terms.append(t)
-        L.append(f"    Mp[{MSLOT[n]}] += " + " + ".join(terms) + ";")
+        L.append(f"    Mp[{MSLOT[n]}] += s{idx[n]};")
     L.append("}")
     return L
 

@@ -352,10 +352,194 @@ __device__ __forceinline__ float bm_d32(const float4 v, float px, float py, floa
 // within twice that margin of the largest FP32 distance is a candidate for the farthest one.
 __device__ __forceinline__ float bm_threshold(float top) { return top - (4e-7f + 6e-7f * top); }
 
-#ifndef FMM_UPWARD_MINB
-#define FMM_UPWARD_MINB 5  // resident blocks per SM the upward pass is compiled for (96 registers; 4: 128)
-#endif
-__global__ void __launch_bounds__(128, FMM_UPWARD_MINB) k_upward(const unsigned int* __restrict__ nbucket, const int* __restrict__ bucket_cell,
+// The arrival at a parent: publishes this warp's stores before it (those of the other lanes through the
+// warp barrier before the call) and, for the second to arrive, makes the sibling's visible after it.
+__device__ __forceinline__ unsigned int arrive_acq_rel(unsigned int* a)
+{
+    unsigned int old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(a) : "memory");
+    return old;
+}
+
+// Centre of mass and mass of a cell from its two children's.
+__device__ __forceinline__ Com4 parent_com(const Com4& a0, const Com4& a1)
+{
+    const double M = __dadd_rn(a0.w, a1.w), iM = 1.0 / M;  // one FP64 division (a software sequence) instead of three
+    return make_com4(__dmul_rn(__fma_rn(a0.w, a0.x, __dmul_rn(a1.w, a1.x)), iM),
+                     __dmul_rn(__fma_rn(a0.w, a0.y, __dmul_rn(a1.w, a1.y)), iM),
+                     __dmul_rn(__fma_rn(a0.w, a0.z, __dmul_rn(a1.w, a1.z)), iM), M);
+}
+
+// The cell arrays that the upward pass reads and writes.
+struct UpCells {
+    const int *cparent, *cchild;
+    Com4* com;
+    double *clo, *chi;
+    int* cnact;
+    float* rec;
+};
+
+// Cell p from its two children, by one thread.
+__device__ __forceinline__ void up_cell_thread(const UpCells& u, int p, int c0, int c1)
+{
+    const Com4 a0 = ldcg_d4(&u.com[c0]), a1 = ldcg_d4(&u.com[c1]), P = parent_com(a0, a1);
+    float Mq[FMM_NMOM];
+#pragma unroll
+    for (int i = 0; i < FMM_NMOM; i++) Mq[i] = 0.0f;
+    for (int h = 0; h < 2; h++) {
+        const Com4 ac = h ? a1 : a0;
+        float Mc[FMM_NMOM];
+        const float* src = u.rec + (long long)(h ? c1 : c0) * FMM_NREC;
+#pragma unroll
+        for (int i = 0; i < FMM_NMOM; i++) Mc[i] = __ldcg(src + i);
+        fmm_m2m_acc(Mc, fmm_d2f_rn(__dsub_rn(ac.x, P.x)), fmm_d2f_rn(__dsub_rn(ac.y, P.y)),
+                    fmm_d2f_rn(__dsub_rn(ac.z, P.z)), Mq);
+    }
+    u.com[p] = P;
+    for (int a = 0; a < 3; a++) {
+        u.clo[3 * p + a] = fmm_dfrom(min(fmm_nonneg_key(__ldcg(&u.clo[3 * c0 + a])), fmm_nonneg_key(__ldcg(&u.clo[3 * c1 + a]))));
+        u.chi[3 * p + a] = fmm_dfrom(max(fmm_nonneg_key(__ldcg(&u.chi[3 * c0 + a])), fmm_nonneg_key(__ldcg(&u.chi[3 * c1 + a]))));
+    }
+    u.cnact[p] = __ldcg(&u.cnact[c0]) + __ldcg(&u.cnact[c1]);
+    write_record(u.rec + (long long)p * FMM_NREC, Mq);
+}
+
+// The same by a whole warp, half of it per child: three of the 35 moments to order 4 per lane, shifted
+// along one axis after the other as fmm_m2m_acc does, operation for operation, so that the cell has
+// the same bits (its terms past the power are products with zero).
+struct UpWarp {
+    float4 term[2][3][5];   // per child, axis and power a: C(a, i) t^i for i = 1..4
+    float m[2][2][36];      // per child, two rows of the moments; the last stays zero
+    float s[FMM_NREC];      // the parent's record
+};
+
+// For moment q (of 35), per axis: the indices of the moments 1..4 powers lower, six bits each (35: none),
+// and the power above them
+__device__ __forceinline__ void up_shift_index(int q, unsigned int idx[3])
+{
+    int o = 0, m = 0;
+    while (o < 4 && q >= (o + 1) * (o + 2) * (o + 3) / 6) o++;
+    const int r = q - o * (o + 1) * (o + 2) / 6;
+    while (r >= (m + 1) * (m + 2) / 2) m++;
+    const int c = r - m * (m + 1) / 2, n[3] = {o - m, m - c, c};
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        unsigned int w = q < 35 ? (unsigned int)n[a] << 24 : 0u;
+#pragma unroll
+        for (int i = 1; i <= 4; i++) {
+            const int oo = o - i, mm = a == 0 ? m : m - i, cc = a == 2 ? c - i : c;
+            const bool in = q < 35 && n[a] >= i;
+            w |= (unsigned int)(in ? oo * (oo + 1) * (oo + 2) / 6 + mm * (mm + 1) / 2 + cc : 35) << (6 * (i - 1));
+        }
+        idx[a] = w;
+    }
+}
+
+// What a lane does in up_cell_warp, prepared once: its moments' indices, and its up to four terms
+// (position in W.term[h], axis and i of x = hl + 16 k < 60; binomial, 0 past the power)
+struct UpLane {
+    unsigned int idx[3][3];
+    float binom[4];
+    int what[4];  // axis | (i - 1) << 2, -1: none
+};
+
+__device__ __forceinline__ void up_lane(UpLane& U, int hl)
+{
+#pragma unroll
+    for (int k = 0; k < 3; k++) up_shift_index(hl + 16 * k, U.idx[k]);
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int x = hl + 16 * k, axis = x / 20, a = (x % 20) >> 2, i = x & 3;
+        // binomials C(a, i) of a = 1..4, four bits each, from i = 1 up
+        U.binom[k] = a == 0 ? 0.0f : (float)((int)(0x1464013300120001ull >> (16 * (a - 1) + 4 * i)) & 15);
+        U.what[k] = x < 60 ? axis | i << 2 : -1;
+    }
+}
+
+__device__ __forceinline__ void up_cell_warp(const UpCells& u, int p, int c0, int c1, UpWarp& W, const UpLane& U, int lane)
+{
+    const int h = lane >> 4, hl = lane & 15, ch = h ? c1 : c0;
+    // everything this cell needs, in one round of loads
+    const Com4 a0 = ldcg_d4(&u.com[c0]), a1 = ldcg_d4(&u.com[c1]);
+    const float* src = u.rec + (long long)ch * FMM_NREC;
+    float v[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int q = hl + 16 * k;
+        v[k] = q == 0 ? __ldcg(src) : q >= 4 && q < 35 ? __ldcg(src + q - 3) : 0.0f;
+    }
+    double e0 = 0.0, e1 = 0.0;  // box: lanes 0..2 the low side of an axis, 3..5 the high side
+    int n0 = 0;
+    if (lane < 6) {
+        const double* box = lane < 3 ? u.clo : u.chi;
+        const int a = lane < 3 ? lane : lane - 3;
+        e0 = __ldcg(&box[3 * c0 + a]);
+        e1 = __ldcg(&box[3 * c1 + a]);
+    } else if (lane == 6) {
+        n0 = __ldcg(&u.cnact[c0]) + __ldcg(&u.cnact[c1]);
+    }
+    const Com4 P = parent_com(a0, a1), ac = h ? a1 : a0;
+    const float t[3] = {fmm_d2f_rn(__dsub_rn(ac.x, P.x)), fmm_d2f_rn(__dsub_rn(ac.y, P.y)), fmm_d2f_rn(__dsub_rn(ac.z, P.z))};
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int axis = U.what[k] & 3, i = U.what[k] >> 2;
+        const float t1 = axis == 0 ? t[0] : axis == 1 ? t[1] : t[2];
+        const float t2 = __fmul_rn(t1, t1), t3 = __fmul_rn(t2, t1), t4 = __fmul_rn(t3, t1);
+        const float pw = i == 0 ? t1 : i == 1 ? t2 : i == 2 ? t3 : t4;
+        if (U.what[k] >= 0)
+            reinterpret_cast<float*>(W.term[h])[hl + 16 * k] = U.binom[k] != 0.0f ? __fmul_rn(U.binom[k], pw) : 0.0f;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        float* const row = W.m[h][a & 1];
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+            if (hl + 16 * k < 35) row[hl + 16 * k] = v[k];
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            const unsigned int w = U.idx[k][a];
+            const float4 f = W.term[h][a][w >> 24];
+            v[k] = fmaf(f.x, row[w & 63u], v[k]);
+            v[k] = fmaf(f.y, row[(w >> 6) & 63u], v[k]);
+            v[k] = fmaf(f.z, row[(w >> 12) & 63u], v[k]);
+            v[k] = fmaf(f.w, row[(w >> 18) & 63u], v[k]);
+        }
+    }
+    // the children's sum (0 + first + second, as one thread adds them), then the traces of the record
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const float w = __shfl_xor_sync(FMM_FULL_MASK, v[k], 16);
+        const int q = hl + 16 * k;
+        if (h == 0 && q < 35 && (q == 0 || q >= 4)) W.s[q == 0 ? 0 : q - 3] = __fadd_rn(__fadd_rn(0.0f, v[k]), w);
+    }
+    __syncwarp();
+    if (lane == 0) fmm_moment_traces(W.s);
+    __syncwarp();
+    float* const dst = u.rec + (long long)p * FMM_NREC;
+    dst[lane] = W.s[lane];
+    if (lane < FMM_NREC - 32) dst[lane + 32] = W.s[lane + 32];
+    if (lane < 3) u.clo[3 * p + lane] = fmm_dfrom(min(fmm_nonneg_key(e0), fmm_nonneg_key(e1)));
+    else if (lane < 6) u.chi[3 * p + lane - 3] = fmm_dfrom(max(fmm_nonneg_key(e0), fmm_nonneg_key(e1)));
+    else if (lane == 6) u.cnact[p] = n0;
+    else if (lane == 7) u.com[p] = P;
+    __syncwarp();
+}
+
+// The upward pass.  A thread per bucket takes the bucket's sums and moments, then climbs.  It is bound by
+// latency: of a lone warp's 10,500 cycles per level, 1600 were the arrival's fences and atomic, 1600 the
+// tree's links and then the children's records, 1000 the FP64 centre (the division above all), the
+// rest one thread's 700 instructions; and the bucket's two loops waited 1200 cycles for each particle.
+// So the particles are loaded four at a time, the links during the arrival, the arrival is one
+// acquire-release atomic, and where at most UP_COOP lanes of a warp go on, the warp computes their
+// cells together.  Tree phase before and after: 4096 particles 0.284 to 0.259 ms, 63^3 0.605 to 0.558,
+// 128^3 1.30 to 1.19, dual-tree substep 0.646 to 0.605, 384^3 26.0 to 25.7.  (UP_COOP 4: 0.275 ms on the
+// 4096-particle box, 8: 0.31.  5 blocks per SM, 96 registers with spills: 1.22 ms on the 128^3 box, 25.5 on
+// the 384^3 one.)
+#define UP_COOP 2
+#define UP_THREADS 128
+#define FMM_UPWARD_MINB 4
+__global__ void __launch_bounds__(UP_THREADS, FMM_UPWARD_MINB) k_upward(const unsigned int* __restrict__ nbucket, const int* __restrict__ bucket_cell,
                                                 const int* __restrict__ cfirst, const int* __restrict__ ccount,
                                                 const int* __restrict__ cparent, const int* __restrict__ cchild,
                                                 const double* __restrict__ sx, const double* __restrict__ sy,
@@ -365,104 +549,136 @@ __global__ void __launch_bounds__(128, FMM_UPWARD_MINB) k_upward(const unsigned 
                                                 double* chi, double* bmax, int* cnact, float* rec,
                                                 float4* __restrict__ off, unsigned int* arrive)
 {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= (int)*nbucket) return;
-    int c = bucket_cell[b];
-    int f = cfirst[c], cnt = ccount[c];
-    // FP64 issues at 1/64 of the FP32 rate here: the sums stay FP64, while the box is a minimum and
-    // maximum of the positions' order keys, the widening of the mass and the rounding of the offsets
-    // work on the encodings (f64bits.cuh), and the exact squared distances are evaluated only for
-    // the particles that can be the farthest
-    double M = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
-    unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
-    int na = 0;
-    for (int j = f; j < f + cnt; j++) {
-        double m = fmm_f2d(sm[j]), x = sx[j], y = sy[j], z = sz[j];
-        M += m;
-        mx += m * x;
-        my += m * y;
-        mz += m * z;
-        const unsigned long long kx = fmm_nonneg_key(x), ky = fmm_nonneg_key(y), kz = fmm_nonneg_key(z);
-        lo[0] = min(lo[0], kx);
-        hi[0] = max(hi[0], kx);
-        lo[1] = min(lo[1], ky);
-        hi[1] = max(hi[1], ky);
-        lo[2] = min(lo[2], kz);
-        hi[2] = max(hi[2], kz);
-        na += sact[j] ? 1 : 0;
-    }
-    const double iM = 1.0 / M;  // one FP64 division (a software sequence on this part) instead of three
-    double cx = mx * iM, cy = my * iM, cz = mz * iM;
-    float Mo[FMM_NMOM];
+    __shared__ UpWarp warps[UP_THREADS / 32];
+    const int b = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    UpWarp& W = warps[threadIdx.x >> 5];
+    const UpCells u = {cparent, cchild, com, clo, chi, cnact, rec};
+    int p = -1;  // the cell this lane climbs to
+    if (b < (int)*nbucket) {
+        const int c = bucket_cell[b];
+        const int f = cfirst[c], cnt = ccount[c];
+        // FP64 issues at 1/64 of the FP32 rate here: the sums stay FP64, while the box is a minimum and
+        // maximum of the positions' order keys, the widening of the mass and the rounding of the offsets
+        // work on the encodings (f64bits.cuh), and the exact squared distances are evaluated only for
+        // the particles that can be the farthest
+        double M = 0.0, mx = 0.0, my = 0.0, mz = 0.0;
+        unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
+        int na = 0;
+        for (int j0 = f; j0 < f + cnt; j0 += 4) {
+            double xs[4], ys[4], zs[4];
+            float ms[4];
+            unsigned char as[4];
 #pragma unroll
-    for (int i = 0; i < FMM_NMOM; i++) Mo[i] = 0.0f;
-    // the FP32 distances from the rounded centre single out the candidates for the farthest particle
-    // (the margin of the exact b_max passes below), at most 32 of them in a bit mask
-    const float pcx = fmm_d2f_rn(cx), pcy = fmm_d2f_rn(cy), pcz = fmm_d2f_rn(cz);
-    float m2 = 0.0f;
-    for (int j = f; j < f + cnt; j++) {
-        double dx = sx[j] - cx, dy = sy[j] - cy, dz = sz[j] - cz;
-        float m = sm[j];
-        float fx = fmm_d2f_rn(dx), fy = fmm_d2f_rn(dy), fz = fmm_d2f_rn(dz);
-        fmm_p2m_acc(m, fx, fy, fz, Mo);
-        off[j] = make_float4(fx, fy, fz, m);
-        m2 = fmaxf(m2, bm_d2_32(posf[j], pcx, pcy, pcz));
-    }
-    const float thr = bm_threshold(sqrtf(m2));
-    double b2 = 0.0;
-    for (int j0 = f; j0 < f + cnt; j0 += 32) {
-        unsigned int cand = 0u;
-        for (int t = 0; t < 32 && j0 + t < f + cnt; t++)
-            if (bm_d32(posf[j0 + t], pcx, pcy, pcz) >= thr) cand |= 1u << t;
-        while (cand) {
-            const int j = j0 + __ffs(cand) - 1;
-            cand &= cand - 1;
-            b2 = fmax(b2, dist2_ordered(sx[j] - cx, sy[j] - cy, sz[j] - cz));
+            for (int k = 0; k < 4; k++) {
+                const int j = min(j0 + k, f + cnt - 1);
+                xs[k] = sx[j];
+                ys[k] = sy[j];
+                zs[k] = sz[j];
+                ms[k] = sm[j];
+                as[k] = sact[j];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (j0 + k >= f + cnt) break;
+                const double m = fmm_f2d(ms[k]), x = xs[k], y = ys[k], z = zs[k];
+                M += m;
+                mx += m * x;
+                my += m * y;
+                mz += m * z;
+                const unsigned long long kx = fmm_nonneg_key(x), ky = fmm_nonneg_key(y), kz = fmm_nonneg_key(z);
+                lo[0] = min(lo[0], kx);
+                hi[0] = max(hi[0], kx);
+                lo[1] = min(lo[1], ky);
+                hi[1] = max(hi[1], ky);
+                lo[2] = min(lo[2], kz);
+                hi[2] = max(hi[2], kz);
+                na += as[k] ? 1 : 0;
+            }
         }
-    }
-    com[c] = make_com4(cx, cy, cz, M);
-    for (int a = 0; a < 3; a++) {
-        clo[3 * c + a] = fmm_dfrom(lo[a]);
-        chi[3 * c + a] = fmm_dfrom(hi[a]);
-    }
-    bmax[c] = __dsqrt_rn(b2);
-    cnact[c] = na;
-    write_record(rec + (long long)c * FMM_NREC, Mo);
-    // climb: the second child to arrive at a parent computes it
-    int p = cparent[c];
-    while (p >= 0) {
-        __threadfence();
-        unsigned int old = atomicAdd(&arrive[p], 1u);
-        if (old == 0u) return;
-        __threadfence();
-        int c0 = cchild[2 * p], c1 = cchild[2 * p + 1];
-        Com4 a0 = ldcg_d4(&com[c0]), a1 = ldcg_d4(&com[c1]);
-        double Mp = a0.w + a1.w;
-        const double iMp = 1.0 / Mp;
-        double px = (a0.w * a0.x + a1.w * a1.x) * iMp;
-        double py = (a0.w * a0.y + a1.w * a1.y) * iMp;
-        double pz = (a0.w * a0.z + a1.w * a1.z) * iMp;
-        float Mq[FMM_NMOM];
+        const double iM = 1.0 / M;  // one FP64 division (a software sequence on this part) instead of three
+        double cx = mx * iM, cy = my * iM, cz = mz * iM;
+        float Mo[FMM_NMOM];
 #pragma unroll
-        for (int i = 0; i < FMM_NMOM; i++) Mq[i] = 0.0f;
-        for (int h = 0; h < 2; h++) {
-            int ch = h ? c1 : c0;
-            Com4 ac = h ? a1 : a0;
-            float Mc[FMM_NMOM];
-            const float* src = rec + (long long)ch * FMM_NREC;
+        for (int i = 0; i < FMM_NMOM; i++) Mo[i] = 0.0f;
+        // the FP32 distances from the rounded centre single out the candidates for the farthest particle
+        // (the margin of the exact b_max passes below), at most 32 of them in a bit mask
+        const float pcx = fmm_d2f_rn(cx), pcy = fmm_d2f_rn(cy), pcz = fmm_d2f_rn(cz);
+        float m2 = 0.0f;
+        for (int j0 = f; j0 < f + cnt; j0 += 4) {
+            double xs[4], ys[4], zs[4];
+            float4 ps[4];
 #pragma unroll
-            for (int i = 0; i < FMM_NMOM; i++) Mc[i] = __ldcg(src + i);
-            double tx = ac.x - px, ty = ac.y - py, tz = ac.z - pz;
-            fmm_m2m_acc(Mc, fmm_d2f_rn(tx), fmm_d2f_rn(ty), fmm_d2f_rn(tz), Mq);
+            for (int k = 0; k < 4; k++) {
+                const int j = min(j0 + k, f + cnt - 1);
+                xs[k] = sx[j];
+                ys[k] = sy[j];
+                zs[k] = sz[j];
+                ps[k] = posf[j];
+            }
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (j0 + k >= f + cnt) break;
+                const float m = ps[k].w;
+                const float fx = fmm_d2f_rn(xs[k] - cx), fy = fmm_d2f_rn(ys[k] - cy), fz = fmm_d2f_rn(zs[k] - cz);
+                fmm_p2m_acc(m, fx, fy, fz, Mo);
+                off[j0 + k] = make_float4(fx, fy, fz, m);
+                m2 = fmaxf(m2, bm_d2_32(ps[k], pcx, pcy, pcz));
+            }
         }
-        com[p] = make_com4(px, py, pz, Mp);
+        const float thr = bm_threshold(sqrtf(m2));
+        double b2 = 0.0;
+        for (int j0 = f; j0 < f + cnt; j0 += 32) {
+            unsigned int cand = 0u;
+            for (int t = 0; t < 32 && j0 + t < f + cnt; t++)
+                if (bm_d32(posf[j0 + t], pcx, pcy, pcz) >= thr) cand |= 1u << t;
+            while (cand) {
+                const int j = j0 + __ffs(cand) - 1;
+                cand &= cand - 1;
+                b2 = fmax(b2, dist2_ordered(sx[j] - cx, sy[j] - cy, sz[j] - cz));
+            }
+        }
+        com[c] = make_com4(cx, cy, cz, M);
         for (int a = 0; a < 3; a++) {
-            clo[3 * p + a] = fmm_dfrom(min(fmm_nonneg_key(__ldcg(&clo[3 * c0 + a])), fmm_nonneg_key(__ldcg(&clo[3 * c1 + a]))));
-            chi[3 * p + a] = fmm_dfrom(max(fmm_nonneg_key(__ldcg(&chi[3 * c0 + a])), fmm_nonneg_key(__ldcg(&chi[3 * c1 + a]))));
+            clo[3 * c + a] = fmm_dfrom(lo[a]);
+            chi[3 * c + a] = fmm_dfrom(hi[a]);
         }
-        cnact[p] = __ldcg(&cnact[c0]) + __ldcg(&cnact[c1]);
-        write_record(rec + (long long)p * FMM_NREC, Mq);
-        p = cparent[p];
+        bmax[c] = __dsqrt_rn(b2);
+        cnact[c] = na;
+        write_record(rec + (long long)c * FMM_NREC, Mo);
+        p = cparent[c];
+    }
+    // Climb: the second child to arrive at a parent computes it.
+    UpLane U;
+    bool ready = false;
+    for (;;) {
+        // the tree's links do not depend on the children's results: on their way during the arrival
+        int next = -1, c0 = -1, c1 = -1;
+        if (p >= 0) {
+            next = cparent[p];
+            c0 = cchild[2 * p];
+            c1 = cchild[2 * p + 1];
+        }
+        __syncwarp();  // every lane's stores come before the arrival that publishes them
+        if (p >= 0 && arrive_acq_rel(&arrive[p]) == 0u) p = -1;
+        unsigned int todo = __ballot_sync(FMM_FULL_MASK, p >= 0);
+        if (!todo) break;
+        if (__popc(todo) > UP_COOP) {
+            if (p >= 0) up_cell_thread(u, p, c0, c1);
+        } else {
+            if (!ready) {
+                ready = true;
+                up_lane(U, lane & 15);
+                if (lane < 4) W.m[lane >> 1][lane & 1][35] = 0.0f;
+                __syncwarp();
+            }
+            while (todo) {
+                const int q = __ffs(todo) - 1;
+                todo &= todo - 1;
+                up_cell_warp(u, __shfl_sync(FMM_FULL_MASK, p, q), __shfl_sync(FMM_FULL_MASK, c0, q),
+                             __shfl_sync(FMM_FULL_MASK, c1, q), W, U, lane);
+            }
+        }
+        if (p >= 0) p = next;
     }
 }
 
@@ -732,7 +948,7 @@ cudaError_t fmm_launch_upward(DevTree& t, long long n, int bucket, DevCounters* 
     k_bucket_cells<<<(unsigned)fmm_ceil_div(nc, TB), TB, 0, s>>>(t.cfirst, t.cchild, t.dcount, t.bucket_of,
                                                                  t.bucket_cell);
     cudaMemsetAsync(t.arrive, 0, sizeof(unsigned int) * (size_t)nc, s);
-    k_upward<<<(unsigned)fmm_ceil_div(nb, 128), 128, 0, s>>>(t.dcount + 1, t.bucket_cell, t.cfirst, t.ccount,
+    k_upward<<<(unsigned)fmm_ceil_div(nb, UP_THREADS), UP_THREADS, 0, s>>>(t.dcount + 1, t.bucket_cell, t.cfirst, t.ccount,
                                                               t.cparent, t.cchild, t.sx, t.sy, t.sz, t.sm, t.sact,
                                                               t.posf, t.com, t.clo, t.chi, t.bmax, t.cnact, t.rec, t.off,
                                                               t.arrive);
