@@ -684,48 +684,54 @@ __global__ void __launch_bounds__(FRONT_TILE) k_front_place(int level, const Wal
 // Centres enter as float pairs (cen_diff): the sink's (hk, lk), a cell's from cen, a particle's
 // from posf (hi, and its mass) and plo (lo); a source in a periodic copy has its pair shifted
 // (cen_shift) by the copy's integer offset.
-// KIND 0: a cell of several particles (M2L); KIND 1: a particle, or a cell of one (P2L).
-template <int KIND>
-__device__ __forceinline__ void local_entry(unsigned int e, const float4& hk, const float4& lk,
-                                            const float4* __restrict__ cen,
-                                            const float4* __restrict__ posf, const float4* __restrict__ plo,
-                                            const float* __restrict__ rec, float eps2, int ib, int R, float* acc)
+__device__ __forceinline__ void local_offset(unsigned int e, const float4& hk, const float4& lk, float4& hs, float4& ls,
+                                             int ib, int R, float& rx, float& ry, float& rz)
 {
-    const unsigned int j = entry_index(e, ib);
     const unsigned int q = entry_copy(e, ib);
-    const bool shifted = q != copy_centre(R);
-    int nx = 0, ny = 0, nz = 0;
-    if (shifted) copy_shift(q, R, nx, ny, nz);
-    float4 hs, ls;
-    if (e & FMM_PARTICLE_BIT) {
-        hs = posf[j];
-        ls = plo[j];
-    } else {
-        hs = cen[2 * j];
-        ls = cen[2 * j + 1];
-    }
-    if (shifted) {
+    if (q != copy_centre(R)) {
+        int nx, ny, nz;
+        copy_shift(q, R, nx, ny, nz);
         cen_shift(hs.x, ls.x, (float)nx);
         cen_shift(hs.y, ls.y, (float)ny);
         cen_shift(hs.z, ls.z, (float)nz);
     }
-    const float rx = cen_diff(hk.x, lk.x, hs.x, ls.x), ry = cen_diff(hk.y, lk.y, hs.y, ls.y),
-                rz = cen_diff(hk.z, lk.z, hs.z, ls.z);
-    if (KIND == 1) {
-        // a one-particle cell: its particle (mass = moment M[0]) -> local expansion
-        fmm_p2l_acc((e & FMM_PARTICLE_BIT) ? hs.w : rec[(long long)j * FMM_NREC], rx, ry, rz, eps2, acc);
-    } else {
-        float M[FMM_NMOM];
-        const float4* r4 = reinterpret_cast<const float4*>(rec + (long long)j * FMM_NREC);
+    rx = cen_diff(hk.x, lk.x, hs.x, ls.x);
+    ry = cen_diff(hk.y, lk.y, hs.y, ls.y);
+    rz = cen_diff(hk.z, lk.z, hs.z, ls.z);
+}
+
+// M2L sources of a chunk in shared memory, a row each: the moments, then the centre pair.  Read by a
+// lane per source, a warp's load would touch 32 lines; copied 16 bytes per lane along the records it
+// touches 8 (16 for the centres), and the copies need no registers, so the next chunk's are in flight
+// while this one's sources are evaluated.  Walk phase with this, and with a sink's end known from the
+// next chunk's first sink instead of two more dependent loads: 384^3 box 40.2 to 38.5 ms, batch of 27
+// million particles 12.3 to 11.5, 256^3 substep 13.4 to 13.1, 128^3 NFW box 2.63 to 2.59; smaller
+// boxes take the same time.  L1 prefetches of the next sinks' centres gave nothing more.
+#define M2L_ROW (FMM_NMOM + 12)  // floats: a multiple of 4 that is 4 or 12 mod 16 keeps a quarter warp's reads apart
+static_assert(FMM_NMOM == 32 && M2L_ROW % 4 == 0 && M2L_ROW % 8 != 0, "rows of 16-byte pieces");
+
+__device__ __forceinline__ void copy16_async(float* dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned int)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// entries e of the lanes below cnt
+__device__ __forceinline__ void m2l_stage(unsigned int e, int cnt, const float4* __restrict__ cen,
+                                          const float* __restrict__ rec, int ib, float* row, int lane)
+{
+    const unsigned int j = entry_index(e, ib);
 #pragma unroll
-        for (int q4 = 0; q4 < FMM_NMOM / 4; q4++) {
-            const float4 v = r4[q4];
-            M[4 * q4] = v.x;
-            M[4 * q4 + 1] = v.y;
-            M[4 * q4 + 2] = v.z;
-            M[4 * q4 + 3] = v.w;
-        }
-        fmm_m2l_acc(M, rx, ry, rz, eps2, acc);
+    for (int q = 0; q < 8; q++) {
+        const int s = q * 4 + (lane >> 3);
+        const unsigned int js = __shfl_sync(FMM_FULL_MASK, j, s);
+        if (s < cnt) copy16_async(row + s * M2L_ROW + (lane & 7) * 4, rec + (long long)js * FMM_NREC + (lane & 7) * 4);
+    }
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        const int s = q * 16 + (lane >> 1);
+        const unsigned int js = __shfl_sync(FMM_FULL_MASK, j, s);
+        if (s < cnt) copy16_async(row + s * M2L_ROW + FMM_NMOM + (lane & 1) * 4, cen + 2 * (long long)js + (lane & 1));
     }
 }
 
@@ -757,7 +763,9 @@ __global__ void __launch_bounds__(LOCAL_THREADS, FMM_LOCAL_MINB) k_local_flat(
     float eps2, int ib, int R, int level, DevCounters* __restrict__ ctr)
 {
     __shared__ float red[LOCAL_WPB][32][FMM_NL + 1];
+    __shared__ __align__(16) float stage[KIND == 0 ? LOCAL_WPB : 1][KIND == 0 ? 32 * M2L_ROW : 4];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
+    float* const row = KIND == 0 ? stage[wl] : nullptr;  // M2L: this warp's staged sources
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     if (fmm_overflowed(ctr)) return;
@@ -782,21 +790,60 @@ __global__ void __launch_bounds__(LOCAL_THREADS, FMM_LOCAL_MINB) k_local_flat(
         int carry_sink = -1;
         // entries and sinks are read a chunk ahead: of a chunk's two dependent rounds of loads (they, then
         // the centres and records) one passes behind the chunk before (M2L of a 384^3 box -7%)
-        unsigned int e_next = r0 + lane < r1 ? cc[r0 + lane] : 0u;
+        unsigned int e_next = r0 + lane < r1 ? cc[r0 + lane] : 0u, e_second = 0u;
         int sink_next = r0 + lane < r1 ? cc_sink[r0 + lane] : -1;
+        if (KIND == 0) {  // and the sources' copies too
+            m2l_stage(e_next, (int)min(32LL, r1 - r0), cen, rec, ib, row, lane);
+            e_second = r0 + 32 + lane < r1 ? cc[r0 + 32 + lane] : 0u;
+        }
         for (long long base = r0; base < r1; base += 32) {
             const long long idx = base + lane;
             const bool valid = idx < r1;
             const unsigned int e = e_next;
             const int sink = sink_next;
-            e_next = idx + 32 < r1 ? cc[idx + 32] : 0u;
+            const int ahead = KIND == 0 ? 64 : 32;
+            const unsigned int e_last = idx + ahead < r1 ? cc[idx + ahead] : 0u;
+            e_next = KIND == 0 ? e_second : e_last;
+            e_second = e_last;
             sink_next = idx + 32 < r1 ? cc_sink[idx + 32] : -1;
+            float4 hk = make_float4(0.0f, 0.0f, 0.0f, 0.0f), lk = hk;
+            if (valid) {
+                hk = cen[2 * sink];
+                lk = cen[2 * sink + 1];
+                nent++;
+            }
             float acc[FMM_NL];
 #pragma unroll
             for (int i = 0; i < FMM_NL; i++) acc[i] = 0.0f;
-            if (valid) {
-                local_entry<KIND>(e, cen[2 * sink], cen[2 * sink + 1], cen, posf, plo, rec, eps2, ib, R, acc);
-                nent++;
+            if (KIND == 0) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncwarp();
+                float M[FMM_NMOM];
+                const float4* const src = reinterpret_cast<const float4*>(row + lane * M2L_ROW);
+#pragma unroll
+                for (int q4 = 0; q4 < FMM_NMOM / 4; q4++) {
+                    const float4 v = src[q4];
+                    M[4 * q4] = v.x;
+                    M[4 * q4 + 1] = v.y;
+                    M[4 * q4 + 2] = v.z;
+                    M[4 * q4 + 3] = v.w;
+                }
+                float4 hs = src[FMM_NMOM / 4], ls = src[FMM_NMOM / 4 + 1];
+                __syncwarp();  // the rows are free for the next chunk
+                if (base + 32 < r1) m2l_stage(e_next, (int)min(32LL, r1 - base - 32), cen, rec, ib, row, lane);
+                if (valid) {
+                    float rx, ry, rz;
+                    local_offset(e, hk, lk, hs, ls, ib, R, rx, ry, rz);
+                    fmm_m2l_acc(M, rx, ry, rz, eps2, acc);
+                }
+            } else if (valid) {
+                const unsigned int j = entry_index(e, ib);
+                const bool part = (e & FMM_PARTICLE_BIT) != 0u;
+                float4 hs = part ? posf[j] : cen[2 * j], ls = part ? plo[j] : cen[2 * j + 1];
+                float rx, ry, rz;
+                const float m = part ? hs.w : rec[(long long)j * FMM_NREC];  // a one-particle cell: M[0]
+                local_offset(e, hk, lk, hs, ls, ib, R, rx, ry, rz);
+                fmm_p2l_acc(m, rx, ry, rz, eps2, acc);
             }
 #pragma unroll
             for (int i = 0; i < FMM_NL; i++) red[wl][lane][i] = acc[i];
@@ -804,6 +851,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, FMM_LOCAL_MINB) k_local_flat(
             unsigned int heads = __ballot_sync(FMM_FULL_MASK, valid && (lane == 0 || sink != prev));
             __syncwarp();
             const int nvalid = (int)min(32LL, r1 - base);
+            const int after = __shfl_sync(FMM_FULL_MASK, sink_next, 0);  // the next chunk's first sink (-1: none)
             while (heads) {
                 const int st = __ffs(heads) - 1;
                 heads &= heads - 1;
@@ -816,8 +864,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, FMM_LOCAL_MINB) k_local_flat(
                     if (c1 < FMM_NL) sum1 += red[wl][row][c1];
                 }
                 carry_sink = -1;
-                const long long se = (long long)lcc_off[s_sink] + lcc_len[s_sink];
-                if (base + en < se) {  // the sink's list goes on in the next chunk
+                if (en == nvalid && after == s_sink) {  // the sink's list goes on in the next chunk
                     carry0 = sum0;
                     carry1 = sum1;
                     carry_sink = s_sink;
