@@ -471,7 +471,7 @@ fmm_status fmm_multi_index(int *local_idx, int *moment_idx);
  *
  * fmm_debug_local_side: the walk size, in sinks of the context's previous walk, from which each
  * walk level's local expansions (M2L, P2L, L2L) run on a side stream beside the levels below
- * instead of after the last level (default 2^22; a context's first walk never uses it).  Both
+ * instead of after the last level (by default none does; a context's first walk never uses it).  Both
  * orders give the same bits, since every sink's terms are added in its own list order; 0 takes the
  * side stream whenever the context has walked before, so tests can compare the two.  A negative
  * value restores the default.  Returns FMM_ERR_ARG for ctx == NULL. */

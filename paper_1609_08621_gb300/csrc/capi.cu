@@ -177,15 +177,15 @@ struct fmm_ctx {
     // the tree, join before the groups add them)
     cudaStream_t ew_stream = nullptr;
     cudaEvent_t ew_fork = nullptr, ew_join = nullptr;
-    // the local expansions of each walk level run on a side stream while the walk goes on (a fork
-    // after every level, a join before the groups take their expansions)
+    // the local expansions of each walk level on a side stream while the walk goes on (walk_levels: a
+    // fork after every level, a join before the groups take their expansions)
     cudaStream_t loc_stream = nullptr;
     cudaEvent_t loc_fork = nullptr, loc_join = nullptr;
     // positions of the current call as 32-bit fixed-point coordinates (fmm_compute_forces_i32), else
     // NULL and the call's FP64 positions are used
     const unsigned int* cur_ipos = nullptr;
     // walks of at least this many sinks (previous solve) run the local expansions on a side stream
-    // (fmm_debug_local_side; FMM_LOCAL_SIDE_SINKS by default)
+    // (fmm_debug_local_side; none by default)
     long long side_sinks = -1;
     // test hook (fmm_debug_walk_capacity): the walk's first per-warp scratch and list capacities
     long long dbg_scratch = 0, dbg_list_scale = 0;
@@ -796,18 +796,16 @@ static fmm_status ewald_join(fmm_ctx* c, int terms)
 
 // The walk's levels on the context's stream, and the local expansions of every level.
 //
-// A walk of many sinks (at least FMM_LOCAL_SIDE_SINKS in the context's previous walk) forks each level's
-// expansions onto a side stream as soon as the level's walk kernel ends, to run beside the levels
-// below; the context's stream joins the side stream before the groups take their expansions.
-// There the walk warps leave the FMA pipes idle while they wait on loads.  A smaller walk is bound
-// by its longest chains of dependent steps instead, and kernels running beside it lengthen them:
-// measured on one GB300, the side stream took the 512^3 box's walk phase from 155.6 to 144.8 ms
-// (6.8 M sinks) and the 128^3 NFW box's from 4.1 to 5.2 ms (0.1 M sinks), so a smaller walk runs
-// the expansions after its last level.  Grids follow the previous walk's counts (full persistent
-// grids for the context's first walk).
-#ifndef FMM_LOCAL_SIDE_SINKS
-#define FMM_LOCAL_SIDE_SINKS (1LL << 22)
-#endif
+// By default the expansions follow the walk's last level, as whole passes.  A walk of at least
+// c->side_sinks sinks in the context's previous walk (fmm_debug_local_side) forks each level's onto a side
+// stream as soon as the level's walk kernel ends, to run beside the levels below; the context's stream
+// joins the side stream before the groups take their expansions.  The two slow each other down at
+// every size: a small walk is bound by its longest chains of dependent steps, which kernels beside it
+// lengthen, and a large one fills the GPU with 24 warps per SM, whose caches and registers the M2L
+// blocks then share.  Walk phase after / beside: 128^3 NFW box (0.1 million sinks) 4.1 / 5.2 ms, 256^3
+// substep 13.1 / 15.5, 384^3 box 38.5 / 44.1, 448^3 (4.1 million) 63.4 / 71.7, 512^3 (6.2 million)
+// 100.0 / 113.1.  Grids follow the previous walk's counts (full persistent grids for the context's
+// first walk).
 static fmm_status walk_levels(fmm_ctx* c, WalkArgs& a, int levels)
 {
     DevTree& t = c->t;
@@ -817,7 +815,7 @@ static fmm_status walk_levels(fmm_ctx* c, WalkArgs& a, int levels)
     long long prev_sinks = 0;
     if (prev)
         for (int L = 0; L < FMM_MAX_LEVELS; L++) prev_sinks += c->prev_front[L];
-    const long long side_from = c->side_sinks >= 0 ? c->side_sinks : FMM_LOCAL_SIDE_SINKS;
+    const long long side_from = c->side_sinks >= 0 ? c->side_sinks : LLONG_MAX;
     if (!prev || prev_sinks < side_from) {
         for (int L = 0; L < levels; L++) {
             a.level = L;

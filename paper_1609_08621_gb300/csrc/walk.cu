@@ -20,9 +20,9 @@
 // cell's lists are in a deterministic order whatever the scheduling.
 //
 // The local expansion of a walked cell is L_k = L2L(L_parent) + sum of M2L (CC) and P2L
-// (CP) terms.  A level's local lists are complete when its walk kernel ends, so a large walk runs
-// their M2L and P2L terms and the top-down passes on a side stream while the walk goes on below; a
-// small one runs them after its last level.
+// (CP) terms.  The M2L and P2L terms and the top-down passes follow the walk's last level.  A level's
+// local lists are complete when its walk kernel ends, so they can also run level by level beside the
+// walk (walk_levels).
 #include <limits.h>
 
 #include <algorithm>
