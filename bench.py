@@ -59,8 +59,9 @@ PP_FLOPS = 19.0  # FP32 flops of one PP pair in the kernel (3 sub, 3 fma, 3 mul,
 # - the 512^3 box: bytes per (sink, source) pair of the kernel, from the full-size fixed-theta solve
 #   (k_pc 54,254,844,416 B for 31,659,347,808 PC pairs, k_pp 18,396,550,144 B for 128,335,887,451
 #   PP pairs); a learned solve runs the same kernels over fewer pairs, so its traffic is that rate
-#   times its own pair count.
-NCU_TRAFFIC = {"k_pc": 204893440 + 52785664, "k_pp": 94600448 + 20952576}
+#   times its own pair count (of an earlier version of the kernels, before the walk kept its sinks in
+#   tree order).
+NCU_TRAFFIC = {"k_pc": 204933120 + 53011968, "k_pp": 94973696 + 22656768}
 NCU_TRAFFIC_PER_PAIR_512 = {"k_pc": 54254844416 / 31659347808, "k_pp": 18396550144 / 128335887451}
 NCU_TRAFFIC_PARAMS = (16, 64, 128)
 
@@ -77,7 +78,7 @@ def stored_traffic(workload, n_override, tuning, kernel, stats):
         pairs = int(stats.get("n_pc_pairs" if kernel == "k_pc" else "n_pp_pairs", 0) or 0)
         if pairs > 0:
             return (NCU_TRAFFIC_PER_PAIR_512[kernel] * pairs,
-                    "stored: bytes per pair from an earlier ncu capture of this kernel on the fixed-theta solve of "
+                    "stored: bytes per pair from an ncu capture of an earlier version of this kernel on the fixed-theta solve of "
                     "this box at these settings, times this solve's pairs; not measured in this run")
     return None, "no ncu capture of the current kernel at these settings"
 

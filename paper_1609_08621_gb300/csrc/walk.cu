@@ -1,10 +1,10 @@
 // Checklist walk and local expansions (Sec. 3.1).
 //
-// Sink cells are walked top-down, one tree level per launch.  A warp owns one sink cell k
-// and its checklist: the sources its parent left on the checklist ("remain on the
+// Sink cells are walked top-down, one tree level per launch.  A warp (on a level of few sinks, a
+// block) owns one sink cell k and its checklist: the sources its parent left on the checklist ("remain on the
 // checklist for further consideration by the children of the sink cell") plus, for the
 // root, the root itself.  Each lane takes one entry, evaluates the opening criterion and
-// the warp appends the entry to one of five places with ballot/popc ranks:
+// the warp or block appends the entry to one of five places with ballot/popc ranks:
 //   accept  -> k's local-expansion list (CC for a cell, CP for a particle)
 //   defer   -> the checklist handed to k's children
 //   PC, PP  -> the group's interaction lists (k a group: <= g particles)
