@@ -250,8 +250,8 @@ __global__ void __launch_bounds__(GR_THREADS) k_mlp_grad(const float* __restrict
     }
 }
 
-// Adds the blocks' sums in order, compensated: the gradient, written to grad, or taken at once by an Adam step on the
-// trainable weights (bias-corrected moments).
+// Adds the blocks' sums in order, each addition rounded to FP32: the gradient, written to grad, or taken at once by an
+// Adam step on the trainable weights (bias-corrected moments).
 struct AdamArgs {
     float *p, *m, *v;
     float lr, b1, b2, eps, c1, c2;
@@ -262,14 +262,9 @@ __global__ void __launch_bounds__(64) k_mlp_step(const float* __restrict__ part,
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= MLP_NW) return;
-    float gi = 0.0f, lost = 0.0f;  // the sum and its rounding errors (Knuth's two-sum)
+    float gi = 0.0f;
 #pragma unroll 16
-    for (int b = 0; b < nb; b++) {
-        const float x = part[(long long)b * MLP_PART + i], t = gi + x, y = t - gi;
-        lost += (gi - (t - y)) + (x - y);
-        gi = t;
-    }
-    gi += lost;
+    for (int b = 0; b < nb; b++) gi += part[(long long)b * MLP_PART + i];
     if (!ADAM) {
         grad[i] = gi;
         return;
