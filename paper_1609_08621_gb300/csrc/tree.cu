@@ -660,6 +660,7 @@ __global__ void __launch_bounds__(UP_THREADS, FMM_UPWARD_MINB) k_upward(const un
         }
         __syncwarp();  // every lane's stores come before the arrival that publishes them
         if (p >= 0 && arrive_acq_rel(&arrive[p]) == 0u) p = -1;
+        __syncwarp();  // what one lane has acquired, every lane may read (a ballot orders no memory)
         unsigned int todo = __ballot_sync(FMM_FULL_MASK, p >= 0);
         if (!todo) break;
         if (__popc(todo) > UP_COOP) {
