@@ -611,18 +611,14 @@ __global__ void __launch_bounds__(ITHREADS) k_l2p_out(const Group* __restrict__ 
     }
 }
 
-// The output records of the active particles, in the caller's order, into the caller's arrays.  With
-// several boxes the records start as all ones (marked), and those still so are of particles that no
-// sink held.
-__global__ void k_out_split(const float4* __restrict__ out, const unsigned char* __restrict__ active, bool marked,
-                            long long n, float* __restrict__ acc, float* __restrict__ pot,
-                            const DevCounters* __restrict__ ctr)
+// The output records of the active particles, in the caller's order, into the caller's arrays.
+__global__ void k_out_split(const float4* __restrict__ out, const unsigned char* __restrict__ active, long long n,
+                            float* __restrict__ acc, float* __restrict__ pot, const DevCounters* __restrict__ ctr)
 {
     if (fmm_overflowed(ctr)) return;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || (active && active[i] == 0)) return;
     const float4 v = out[i];
-    if (marked && (__float_as_uint(v.x) & __float_as_uint(v.y) & __float_as_uint(v.z) & __float_as_uint(v.w)) == ~0u) return;
     acc[i] = v.x;
     acc[n + i] = v.y;
     acc[2 * n + i] = v.z;
@@ -780,18 +776,13 @@ cudaError_t fmm_launch_l2p_out(DevTree& t, DevWalk& w, DevCounters* ctr, const I
     float4* const out = !perm && n >= FMM_OUT_RECORDS && 4 * n_active >= n ? reinterpret_cast<float4*>(t.radix) : nullptr;
     if (!perm) perm = t.idx;
     const long long ng = t.cap_grid ? w.cap_groups : w.n_groups;
-    const bool marked = t.nbox > 1;
-    if (out && marked) {
-        const cudaError_t e = cudaMemsetAsync(out, 0xff, sizeof(float4) * (size_t)n, s);
-        if (e != cudaSuccess) return e;
-    }
     auto kernel = a.accumulate == 1 ? k_l2p_out<double> : k_l2p_out<float>;
     kernel<<<grid_for(ng), ITHREADS, 0, s>>>(w.groups, &ctr->n_groups, w.cap_groups, w.cap_item_pp, w.cap_item_pc, t.cen,
                                              t.bucket_of, t.bucket_cell, t.off, w.Lg, w.cnt_pp, w.base_pp, w.part_pp,
                                              w.cnt_pc, w.base_pc, w.part_pc, t.act, t.cnact, perm, n, acc, pot, terms,
                                              out, ctr);
     if (out) {
-        k_out_split<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(out, active, marked, n, acc, pot, ctr);
+        k_out_split<<<(unsigned)fmm_ceil_div(n, 256), 256, 0, s>>>(out, active, n, acc, pot, ctr);
         t.n_launches += 1;
     }
     return cudaGetLastError();

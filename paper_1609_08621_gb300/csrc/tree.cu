@@ -124,6 +124,9 @@ __device__ __forceinline__ int delta(const unsigned long long* __restrict__ k, c
     return base + 64 + __clz((unsigned int)(i ^ (int)j));
 }
 
+// Mark of a node with particles of several boxes, in the last particle of its range (n < 2^31).
+#define NODE_BOXES ((int)0x80000000u)
+
 __global__ void k_radix_tree(const unsigned long long* __restrict__ key, const unsigned long long* __restrict__ box,
                              int n, int* __restrict__ ifirst,
                              int* __restrict__ ilast, int* __restrict__ ileft, int* __restrict__ iright,
@@ -152,7 +155,7 @@ __global__ void k_radix_tree(const unsigned long long* __restrict__ key, const u
     int left = (first == gamma) ? (n - 1 + gamma) : gamma;
     int right = (last == gamma + 1) ? (n - 1 + gamma + 1) : gamma + 1;
     ifirst[i] = first;
-    ilast[i] = last;
+    ilast[i] = box && dnode < 8 ? last | NODE_BOXES : last;
     ileft[i] = left;
     iright[i] = right;
     nparent[left] = i;
@@ -162,7 +165,7 @@ __global__ void k_radix_tree(const unsigned long long* __restrict__ key, const u
 
 __device__ __forceinline__ int node_count(const int* ifirst, const int* ilast, int n, int x)
 {
-    return x < n - 1 ? ilast[x] - ifirst[x] + 1 : 1;
+    return x < n - 1 ? (ilast[x] & ~NODE_BOXES) - ifirst[x] + 1 : 1;
 }
 
 // first index of a sorted key array k[0, n) that is >= v
@@ -208,11 +211,13 @@ __global__ void k_split(const int* __restrict__ ifirst, const int* __restrict__ 
     split[x] = (unsigned char)f;
 }
 
-// a node's children are cells when it splits: more than b particles, or the graded flag
+// a node's children are cells when it splits: more than b particles, or particles of several boxes (every
+// box has a root cell of its own, however few particles it and its neighbours hold), or the graded flag
 __device__ __forceinline__ bool node_splits(const int* ifirst, const int* ilast, int n, int bucket,
                                             const unsigned char* split, int x)
 {
-    return split ? (split[x] & 1u) != 0u : node_count(ifirst, ilast, n, x) > bucket;
+    return split ? (split[x] & 1u) != 0u
+                 : node_count(ifirst, ilast, n, x) > bucket || (x < n - 1 && (ilast[x] & NODE_BOXES) != 0);
 }
 
 __global__ void k_keep(const int* __restrict__ ifirst, const int* __restrict__ ilast, const int* __restrict__ nparent,
