@@ -275,7 +275,7 @@ static std::vector<void*> tree_walk_buffers(const fmm_ctx* c)
             t.ccount, t.cparent, t.cchild, t.cnact, t.bucket_cell, t.arrive, t.com, t.clo, t.chi, t.bmax, t.rec,
             t.node, t.mnorm, t.amin, t.bm_cnt, t.bm_base, t.bm32, t.bm64, t.bm_item, t.bm_imax, t.bm_order, t.bm_bin, t.bm_binbase, t.L, t.scan_part,
             t.hist, t.box_off, t.box_root, t.sbox, t.key_orig, t.split, t.nogroup, t.ewald_L, t.cshift, t.pshift,
-            w.f_cell[0], w.f_cell[1], w.f_cloff[0], w.f_cloff[1], w.f_cllen[0], w.f_cllen[1], w.lcc_off, w.lcc_len,
+            w.f_cell[0], w.f_cell[1], w.f_cloff[0], w.f_cloff[1], w.f_cllen[0], w.f_cllen[1], w.front_part, w.lcc_off, w.lcc_len,
             w.lcp_off, w.lcp_len, w.wcells, w.cp, w.cp_sink, w.Lg, w.cnt_pp, w.cnt_pc, w.base_pp, w.base_pc, w.item_pp, w.item_pc, w.part_pp, w.part_pc,
             w.cl[0], w.cl[1], w.pp, w.pc, w.cc, w.cc_sink, w.groups, w.scratch,
             f.cfirst, f.ccount, f.cchild, f.cparent, f.bucket_cell, f.com, f.clo, f.chi, f.bmax, f.rec, f.posf, f.plo,
@@ -675,6 +675,7 @@ static fmm_status ensure_walk(fmm_ctx* c, long long n, int group, const WalkNeed
             CK(alloc(&w.f_cloff[i], need_front));
             CK(alloc(&w.f_cllen[i], need_front));
         }
+        CK(alloc(&w.front_part, fmm_ceil_div(need_front, FMM_FRONT_TILE)));
         CK(alloc(&w.lcc_off, need_front));
         CK(alloc(&w.lcc_len, need_front));
         CK(alloc(&w.lcp_off, need_front));

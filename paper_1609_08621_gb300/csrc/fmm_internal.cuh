@@ -118,6 +118,7 @@ struct __align__(16) Group {
 #define FMM_LIST_CHUNK 64  // default list entries per PP / PC work item
 #define FMM_GMAX 64       // sink slots per group
 #define FMM_LOCAL_STEP 4  // walk levels between those whose cells' local expansions are evaluated
+#define FMM_FRONT_TILE 1024  // sinks per tile of an ordered walk's counts (walk.cu)
 #define FMM_MAX_LEVELS 192  // walk levels: tree depth + 1 (63 key bits + 31 position bits at most)
 
 // Device-side counters and status, one per context.
@@ -270,6 +271,7 @@ struct DevWalk {
     int *f_cell[2] = {nullptr, nullptr};
     unsigned long long *f_cloff[2] = {nullptr, nullptr};
     int *f_cllen[2] = {nullptr, nullptr};
+    unsigned int *front_part = nullptr;  // an ordered walk's children per tile of a level's sinks
     // per cell: its local-expansion entries, multipole sources (lcc, list cc) and point sources
     // (lcp, list cp: particles and one-particle cells)
     unsigned long long *lcc_off = nullptr, *lcp_off = nullptr;

@@ -81,7 +81,7 @@ __device__ __forceinline__ float gap_axis(float lo_s, float hi_s, float lo_k, fl
 #define FMM_ORDER_CELLS (1LL << 20)
 #endif
 #define FRONT_BITS 30  // of a frontier entry's length; above them, in an ordered walk, its children
-#define FRONT_TILE 1024
+#define FRONT_TILE FMM_FRONT_TILE
 
 // What a walk level reads and writes (one kernel parameter).
 struct WalkIO {
@@ -1154,9 +1154,7 @@ cudaError_t fmm_launch_walk_level(DevTree& t, DevWalk& w, DevCounters* ctr, cons
     io.f_cell = w.f_cell[cur];
     io.f_cloff = w.f_cloff[cur];
     io.f_cllen = w.f_cllen[cur];
-    // the tiles' counts go to the scans' scratch, which every walk this large has room in
-    io.ordered = (t.cap_grid ? t.cap_cells : t.n_cells) >= FMM_ORDER_CELLS &&
-                 fmm_ceil_div(w.cap_front, FRONT_TILE) <= t.cap_scan_part;
+    io.ordered = (t.cap_grid ? t.cap_cells : t.n_cells) >= FMM_ORDER_CELLS;
     io.cl_cur = w.cl[cur];
     io.f_cell_next = w.f_cell[nxt];
     io.f_cloff_next = w.f_cloff[nxt];
@@ -1216,9 +1214,9 @@ cudaError_t fmm_launch_walk_level(DevTree& t, DevWalk& w, DevCounters* ctr, cons
     }
     if (io.ordered) {
         const unsigned fb = (unsigned)std::min(fmm_ceil_div(w.cap_front, FRONT_TILE), 304LL);
-        k_front_count<<<fb, FRONT_TILE, 0, s>>>(a.level, w.cap_front, io.f_cllen, t.scan_part, ctr);
+        k_front_count<<<fb, FRONT_TILE, 0, s>>>(a.level, w.cap_front, io.f_cllen, w.front_part, ctr);
         k_front_place<<<fb, FRONT_TILE, 0, s>>>(a.level, t.node, io.f_cell, io.f_cloff, io.f_cllen, io.f_cell_next,
-                                                io.f_cloff_next, io.f_cllen_next, w.cap_front, t.scan_part, ctr);
+                                                io.f_cloff_next, io.f_cllen_next, w.cap_front, w.front_part, ctr);
         t.n_launches += 2;
     }
     return cudaGetLastError();
