@@ -73,12 +73,19 @@ __device__ __forceinline__ float gap_axis(float lo_s, float hi_s, float lo_k, fl
 // leaves its children in its own place, and two small kernels count and place them (k_front_count,
 // k_front_place).  In the order in which the sinks before them happened to finish, neighbours drift
 // apart level by level, and their sources, which they share, come from DRAM again each time.  The two
-// launches per level cost a small walk more than the locality gives it.  Whole solve without / with
-// the order: 384^3 box (10 million cells) 173.1 / 171.4 ms, substep of a 256^3 box 31.6 / 31.2, 200^3
-// box with the learned criterion (1.5 million) 28.0 / 27.5, batch of 27 million particles 54.6 / 54.6,
-// 128^3 NFW box (0.4 million cells) 7.52 / 7.67.
+// launches per level cost a small walk more than the locality gives it.  Whole solve without / with the
+// order, by cells: 128^3 NFW box (0.4 million) 7.81 / 8.21 ms, Plummer 6.3 million particles (1.13) 19.83 /
+// 20.07, 12.7 million (2.28) 40.88 / 40.97, NFW 12.7 million (2.31) 41.8 / 42.2, 14.3 million (2.61) 47.4 / 47.4,
+// 16.8 million (3.08) 56.7 / 56.6, Plummer 24 million (4.3) 71.7 / 71.5, a substep of it with a tenth active
+// 43.6 / 42.8, 32 million (5.8) 96.9 / 96.3; in buckets of 8 and 4 the lines cross between 3 and 5 million.
+// The learned criterion's longer queues gain earlier: Plummer 4.2 million particles (0.76) 15.96 / 15.59,
+// 8 million (1.44) 28.8 / 28.1, 16.8 million (3.03) 55.4 / 54.2; NFW 4.2 million (0.78) 17.06 / 17.14, 6.3 million
+// (1.15) 24.31 / 24.25, 8 million (1.47) 29.9 / 30.1, 16.8 million (3.08) 61.6 / 60.9.
 #ifndef FMM_ORDER_CELLS
-#define FMM_ORDER_CELLS (1LL << 20)
+#define FMM_ORDER_CELLS (5LL << 19)
+#endif
+#ifndef FMM_ORDER_CELLS_NET
+#define FMM_ORDER_CELLS_NET (1LL << 20)
 #endif
 #define FRONT_BITS 30  // of a frontier entry's length; above them, in an ordered walk, its children
 #define FRONT_TILE FMM_FRONT_TILE
@@ -1154,7 +1161,7 @@ cudaError_t fmm_launch_walk_level(DevTree& t, DevWalk& w, DevCounters* ctr, cons
     io.f_cell = w.f_cell[cur];
     io.f_cloff = w.f_cloff[cur];
     io.f_cllen = w.f_cllen[cur];
-    io.ordered = (t.cap_grid ? t.cap_cells : t.n_cells) >= FMM_ORDER_CELLS;
+    io.ordered = (t.cap_grid ? t.cap_cells : t.n_cells) >= (a.mode == 1 ? FMM_ORDER_CELLS_NET : FMM_ORDER_CELLS);
     io.cl_cur = w.cl[cur];
     io.f_cell_next = w.f_cell[nxt];
     io.f_cloff_next = w.f_cloff[nxt];
