@@ -761,10 +761,13 @@ cudaError_t fmm_launch_pc(DevTree& t, DevWalk& w, DevCounters* ctr, const Intera
 // From FMM_OUT_RECORDS particles on (their results no longer fit L2), a solve of the caller's own
 // particles writes each result as one 16-byte record in the caller's order and splits the records in a
 // streaming pass: a scattered store costs a DRAM sector whatever its size, and the four arrays cost
-// four of them per particle.  384^3 box 9.1 to 4.7 ms, 64 boxes 3.5 to 2.1; the 128^3 box, within L2, is
-// slower (0.186 to 0.201), and so is a 256^3 substep with a tenth active (0.73 to 0.86), where the
-// streaming pass reads flags and records of every particle: so at least a quarter must be active.
-#define FMM_OUT_RECORDS (1LL << 22)
+// four of them per particle.  The streaming pass reads the flags and records of every particle, so at
+// least a quarter of them must be active.  Output phase, direct stores / records, Plummer boxes: 4.2 million
+// particles, all active 0.340 / 0.352 ms, a quarter 0.211 / 0.233; 5.2 million 0.420 / 0.408 and 0.266 / 0.279;
+// 5.8 million 0.505 / 0.447 and 0.295 / 0.301, with a fifth 0.274 / 0.297, with 0.35 0.322 / 0.301; 8.4 million
+// 0.997 / 0.719 and 0.481 / 0.451, with a tenth 0.361 / 0.429; 16.8 million 2.35 / 1.40 and 1.00 / 0.87, with a
+// tenth 0.70 / 0.83.
+#define FMM_OUT_RECORDS (11LL << 19)
 cudaError_t fmm_launch_l2p_out(DevTree& t, DevWalk& w, DevCounters* ctr, const InteractArgs& a,
                                const unsigned char* active, long long n_active, float* acc, float* pot, long long n,
                                cudaStream_t s, const unsigned int* perm)
