@@ -170,12 +170,49 @@ __global__ void __launch_bounds__(KD_THREADS, 6) k_kick_drift(
     active_next[i] = ((s1 & ((1LL << (R - r)) - 1)) == 0) ? 1 : 0;
 }
 
+// The same with a single rung (the ordinary time step): substep 0 alone, every particle active and on rung 0 from here
+// on, so there is nothing to gather or to decide.  The gathering kernel's barriers and shared memory cost it
+// 8.5 us against 7.1 on 100,000 particles, 64.4 against 62.2 on 2 million and 570 against 561 on 20 million.
+template <bool CLOSING>
+__global__ void __launch_bounds__(KD_THREADS) k_kick_drift_single(double* __restrict__ pos, double* __restrict__ vel,
+                                                                  const float* __restrict__ acc,
+                                                                  unsigned char* __restrict__ rung,
+                                                                  unsigned char* __restrict__ active_next, long long n,
+                                                                  double dt0, double hk, unsigned int* __restrict__ status)
+{
+    const long long i = (long long)blockIdx.x * KD_THREADS + threadIdx.x;
+    if (i >= n) return;
+    double x[3], hc = hk;  // the closing half step is that of the rung so far
+    if (CLOSING) {
+        const int r = rung[i];
+        if (r != 0) hc = pow2_scale(dt0, r + 1);
+    }
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+        const double f = fmm_f2d(acc[a * n + i]);
+        double v = vel[a * n + i];
+        if (CLOSING) v += f * hc;
+        v += f * hk;
+        vel[a * n + i] = v;
+        x[a] = pos[a * n + i] + v * dt0;
+        pos[a * n + i] = x[a];
+    }
+    if (!(fmm_in_unit(x[0]) && fmm_in_unit(x[1]) && fmm_in_unit(x[2]))) atomicOr(status, FMM_DEV_ERR_ARG);
+    rung[i] = 0;
+    active_next[i] = 1;
+}
+
 cudaError_t fmm_launch_kick_drift(double* pos, double* vel, const float* acc, unsigned char* rung,
                                   unsigned char* active_next, long long n, double eps, double dt0, int max_rung,
                                   int substep, int closing, DevCounters* ctr, cudaStream_t s)
 {
-    k_kick_drift<<<(unsigned)fmm_ceil_div(n, KD_THREADS), KD_THREADS, 0, s>>>(pos, vel, acc, rung, active_next, n, eps, dt0,
-                                                                max_rung, rung_threshold(eps, dt0), substep, closing, &ctr->status);
+    const unsigned blocks = (unsigned)fmm_ceil_div(n, KD_THREADS);
+    const auto single = closing ? k_kick_drift_single<true> : k_kick_drift_single<false>;
+    if (max_rung == 0)
+        single<<<blocks, KD_THREADS, 0, s>>>(pos, vel, acc, rung, active_next, n, dt0, 0.5 * dt0, &ctr->status);
+    else
+        k_kick_drift<<<blocks, KD_THREADS, 0, s>>>(pos, vel, acc, rung, active_next, n, eps, dt0, max_rung,
+                                                   rung_threshold(eps, dt0), substep, closing, &ctr->status);
     return cudaGetLastError();
 }
 
