@@ -38,8 +38,8 @@ __device__ __noinline__ int target_rung_f64(float ax, float ay, float az, double
 // definition's own roundings within 1e-14, so a square further than 1e-6 from the thresholds on both
 // sides of it has the definition's rung; the others (one particle in about a million) take it.  The
 // FP64 square roots and division (FP64 issues at 1/64 of the FP32 rate, and a warp pays in full for one
-// active lane) made the kick-drift of a 256^3 box with a tenth active 1.62 ms, 0.8 TB/s; it takes
-// 0.46 ms, 2.8 TB/s, this way, bound by the FP64 multiply-adds of the kicks and the drift.
+// active lane) made the kick-drift of a 256^3 box with a tenth active 1.62 ms, 0.8 TB/s; it took
+// 0.46 ms, 2.8 TB/s, this way.
 __device__ __forceinline__ int target_rung(float ax, float ay, float az, double eps, double dt0, int R, float t0)
 {
     if (R == 0) return 0;  // a single rung: nothing to decide
@@ -86,8 +86,9 @@ __device__ __forceinline__ double pow2_scale(double dt0, int k)
 // A warp pays for an FP64 instruction in full however few of its lanes are active, and on a substep
 // nearly every warp holds some of the active tenth.  So a block gathers its active particles in shared
 // memory and kicks them with as few warps as hold them; the drift, of every particle, follows.  256^3 box,
-// a tenth active: 0.365 ms, 4.1 TB/s, against 0.465 with every particle kicked in its own lane (6 blocks per
-// SM; 0.39 with 5, 0.41 with 4).
+// a tenth active: 0.353 ms, 4.2 TB/s, against 0.465 with every particle kicked in its own lane (6 blocks per
+// SM; 0.39 with 5, 0.41 with 4).  Neither pipe alone bounds it: FP64 is busy for 62% of the time and DRAM for
+// 57%, and the warps wait at the barriers, most of all for the accelerations, which are loaded behind one.
 #define KD_THREADS 256
 __global__ void __launch_bounds__(KD_THREADS, 6) k_kick_drift(
     double* __restrict__ pos, double* __restrict__ vel, const float* __restrict__ acc, unsigned char* __restrict__ rung,

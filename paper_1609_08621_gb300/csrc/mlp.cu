@@ -54,7 +54,8 @@ cudaError_t fmm_mlp_pack(const float* params, unsigned char* packed, cudaStream_
 
 // Gradient of 0.5 * mean((y - label)^2) over a minibatch.  A block takes tiles of 64 rows and keeps its
 // weight gradients in registers over them; its sums go to a slot of its own, and k_mlp_step adds the
-// slots in order, so the weights of a training run are a function of its inputs.  (The loss is summed row by row
+// slots in order, so the weights of a training run are a function of its inputs (atomics gave each run another
+// order of arrival from three blocks on, and training turns a rounding into 1e-5 to 6e-3 of the weights).  (The loss is summed row by row
 // with atomics.)
 //
 // The six products of a tile (two hidden layers forward, their deltas, their weight gradients) are
